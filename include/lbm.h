@@ -256,8 +256,9 @@ LBM_API lbm_status lbm_bind_geometry(lbm_plan* plan, const uint32_t* d_link);
  * states); only the plan's workspace and the tables change.
  *
  * lbm_compact_size: bytes of the table buffer for n_fluid fluid nodes
- *   (4 n_fluid dense indices, 4 (Q - 1) n_fluid neighbour codes, one bit per
- *   fluid node, 4 N dense-to-compact map, scan scratch).
+ *   (4 n_fluid dense indices, 4 (Q - 1) n_fluid neighbour codes, one bit and
+ *   4 bytes per fluid node, 16 bytes per 30 columns of every row, 4 N
+ *   dense-to-compact map, scan scratch).
  * lbm_compact_bind: builds the tables from the bound link array into
  *   d_tables (device, caller-owned, 256-byte aligned, lbm_compact_size
  *   bytes, valid while the plan uses it) and switches the plan to the compact

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kStepThreads)
         bool mrt_done = false;
         if constexpr (Q == 9) {
             if (bc.mrt) {
-                domT = adjoint_collision_mrt<T>(f, mu, drho, rho, u, G, omega, mrt_rates(bc.status), lamv);
+                domT = adjoint_collision_mrt<T>(f, mu, drho, rho, u, G, omega, bc.mrt_rates, lamv);
                 mrt_done = true;
             }
         }

@@ -135,35 +135,6 @@ bool aligned256(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 25
 
 unsigned char* bytes(void* ws) { return static_cast<unsigned char*>(ws); }
 
-// The MRT rates and the inlet velocity into the status section, where the
-// kernels read them (Bc::mrt, Bc::vel_inlet).
-struct CallParams {
-    double rates[3], u_in[3];
-};
-
-__global__ void k_write_call_params(uint32_t* status, CallParams c)
-{
-    unsigned char* b = reinterpret_cast<unsigned char*>(status);
-    double* r = reinterpret_cast<double*>(b + kMrtRates);
-    double* u = reinterpret_cast<double*>(b + kInletVelocity);
-    for (int i = 0; i < 3; ++i) {
-        r[i] = c.rates[i];
-        u[i] = c.u_in[i];
-    }
-}
-
-lbm_status write_mrt_rates(const lbm_plan* p, const Bc& bc, cudaStream_t s)
-{
-    if (!p->info.mrt && !p->info.vel_inlet) return LBM_OK;
-    CallParams c;
-    for (int i = 0; i < 3; ++i) {
-        c.rates[i] = p->info.mrt_rates[i];
-        c.u_in[i] = p->info.u_in[i];
-    }
-    k_write_call_params<<<1, 1, 0, s>>>(bc.status, c);
-    return cuda_status(cudaGetLastError());
-}
-
 // The periodic-y and velocity-inlet options exist in the fluid-only layout
 // only; the in-place schedule keeps no neighbour velocity for the
 // extrapolated Eq. 6 velocity.
@@ -187,6 +158,11 @@ Bc make_bc(const lbm_plan* p, const double* rho_in, double rho_out, void* ws)
     bc.wait_us = p->info.wait_us;
     bc.test_stall = p->info.test_stall ? 1 : 0;
     bc.ramp_steps = p->info.vel_inlet ? p->info.ramp_steps : 0;
+    bc.ramp = inlet_ramp(bc.ramp_steps, 0);
+    for (int a = 0; a < 3; ++a) {
+        bc.u_in[a] = p->info.u_in[a];
+        bc.mrt_rates[a] = p->info.mrt_rates[a];
+    }
     return bc;
 }
 
@@ -592,8 +568,11 @@ lbm_status lbm_compact_bind(lbm_plan* p, int64_t n_fluid, void* d_tables, void* 
     Cmp c{0, nullptr, nullptr};
     const int32_t* cmap = nullptr;
     const BCmpInst* inst = nullptr;
-    LBM_TRY(compact_build(p->info, n_fluid, d_tables, &c, &cmap, &inst, static_cast<cudaStream_t>(stream)));
+    BCmpInst host = {};
+    LBM_TRY(compact_build(p->info, n_fluid, d_tables, &c, &cmap, &inst, &host, static_cast<cudaStream_t>(stream)));
     p->info.cmp = c;
+    p->info.cmp_lat = host.lat;
+    p->info.cmp_int = host.n_int;
     p->info.cmp_map = cmap;
     p->info.cmp_inst = inst;
     p->info.state_bytes = (size_t)p->info.q * (size_t)n_fluid * (size_t)p->info.prec;
@@ -667,7 +646,6 @@ lbm_status lbm_forward(lbm_plan* p, const double* d_rho_in, const double* d_tau,
     unsigned char* last = nullptr;
     chain([](const unsigned char*, bool, unsigned char*, unsigned char*, int) { return LBM_OK; }, g0, &last);
     auto issue = [&](cudaStream_t st_) -> lbm_status {
-        LBM_TRY(write_mrt_rates(p, bc, st_));
         if (cudaMemsetAsync(g0, 0, p->info.state_bytes, st_) != cudaSuccess) return LBM_ERR_CUDA;  // g^0 = rest
         if (one && cudaMemsetAsync(bcs.side_u, 0, (size_t)p->info.prec * 6 * (size_t)p->info.n_acc, st_) !=
                        cudaSuccess)
@@ -710,7 +688,6 @@ lbm_status lbm_step(lbm_plan* p, const double* d_rho_in, const double* d_tau, do
     const bool one = in_place(p);
     Bc bcs = bc;
     if (one) bcs.side_u = ws + p->ws.side;  // the collide-only launch writes the Eq. 6 nodes' velocities
-    LBM_TRY(write_mrt_rates(p, bc, s));
     if (p->info.cmp.nf)
         LBM_TRY(step_launch_cmp(p->info, kCollideOnly, d_f_in, ping0, true, false, bcs, tau, s));
     else
@@ -941,7 +918,6 @@ static lbm_status reverse_sweep(lbm_plan* p, const double* d_rho_in, const doubl
         if (cudaMemsetAsync(win->d_loss, 0, sizeof(double), s) != cudaSuccess ||
             cudaMemsetAsync(lam_T, 0, p->info.state_bytes, s) != cudaSuccess)
             return LBM_ERR_CUDA;
-        LBM_TRY(write_mrt_rates(p, bc, s));
         for (int o = 0; o < win->n_obs; ++o)
             if (win->steps[o] == T) LBM_TRY(observe(o, T, nullptr, lam_T, s));
     } else if (p->info.cmp.nf) {  // lambda^T into the compact layout
@@ -950,7 +926,6 @@ static lbm_status reverse_sweep(lbm_plan* p, const double* d_rho_in, const doubl
         return LBM_ERR_CUDA;
     }
     auto issue = [&](cudaStream_t st_) -> lbm_status {
-        LBM_TRY(write_mrt_rates(p, bc, st_));
         lam_cur = lam_T;
         lam_next = 0;
         if (cudaMemsetAsync(grad_acc, 0, sizeof(double) * (size_t)p->info.n_acc, st_) != cudaSuccess)

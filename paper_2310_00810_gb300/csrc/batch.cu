@@ -352,7 +352,6 @@ struct lbm_batch {
     bool cmp = false;
     long long nfp = 0;                 // packed compact nodes (every instance padded to kBatchCmpAlign)
     std::vector<BCmpInst> cinsts;
-    std::vector<int> blk_inst;
     BCmpArgs ca = {};
     size_t cmp_state_bytes = 0;
     struct G {
@@ -807,14 +806,16 @@ lbm_status lbm_batch_adjoint(lbm_batch* b, const double* d_rho_in, const double*
 lbm_status lbm_batch_compact_size(const lbm_batch* b, const int64_t* n_fluid, size_t* bytes)
 {
     if (!b || !n_fluid || !bytes) return LBM_ERR_INVALID_ARG;
-    long long nfp = 0;
+    long long nfp = 0, n_win = 0;
     for (int i = 0; i < b->n; ++i) {
         if (n_fluid[i] < 0 || n_fluid[i] > b->info[i].geo.N) return LBM_ERR_INVALID_ARG;
         nfp += (n_fluid[i] + kBatchCmpAlign - 1) / kBatchCmpAlign * kBatchCmpAlign;
+        n_win += window_count(b->info[(size_t)i]);
     }
-    *bytes = al256(sizeof(BCmpInst) * (size_t)b->n) + al256(sizeof(int) * (size_t)(nfp / kBatchCmpAlign)) +
+    *bytes = al256(sizeof(BCmpInst) * (size_t)b->n) + al256(2 * sizeof(CmpBlk) * (size_t)(nfp / kBatchCmpAlign)) +
              al256(sizeof(int32_t) * (size_t)nfp) + al256(sizeof(int32_t) * (size_t)(b->q - 1) * (size_t)nfp) +
-             al256(sizeof(uint32_t) * (size_t)(nfp / 32));
+             al256(sizeof(uint32_t) * (size_t)(nfp / 32)) + al256(sizeof(uint32_t) * (size_t)nfp) +
+             al256(sizeof(uint2) * (size_t)n_win) + al256(sizeof(int2) * (size_t)n_win);
     return LBM_OK;
 }
 
@@ -848,53 +849,87 @@ lbm_status lbm_batch_compact_bind(lbm_batch* b, const int64_t* n_fluid, void* d_
     if (nfp >= (1LL << 31)) return LBM_ERR_INVALID_ARG;  // neighbour codes are int32
     unsigned char* tb = static_cast<unsigned char*>(d_tables);
     const size_t t_insts = 0, t_blk = al256(sizeof(BCmpInst) * (size_t)b->n);
-    const size_t t_idx = t_blk + al256(sizeof(int) * (size_t)(nfp / kBatchCmpAlign));
+    const size_t t_idx = t_blk + al256(2 * sizeof(CmpBlk) * (size_t)(nfp / kBatchCmpAlign));
     const size_t t_nbr = t_idx + al256(sizeof(int32_t) * (size_t)nfp);
     int32_t* idx = reinterpret_cast<int32_t*>(tb + t_idx);
     int32_t* nbr = reinterpret_cast<int32_t*>(tb + t_nbr);
     const size_t t_eq6 = t_nbr + al256(sizeof(int32_t) * (size_t)(b->q - 1) * (size_t)nfp);
     uint32_t* eq6 = reinterpret_cast<uint32_t*>(tb + t_eq6);
-    std::vector<int> blk((size_t)(nfp / kBatchCmpAlign));
+    long long n_win = 0;
+    for (int i = 0; i < b->n; ++i) n_win += window_count(b->info[(size_t)i]);
+    const size_t t_pos = t_eq6 + al256(sizeof(uint32_t) * (size_t)(nfp / 32));
+    const size_t t_win = t_pos + al256(sizeof(uint32_t) * (size_t)nfp);
+    const size_t t_edge = t_win + al256(sizeof(uint2) * (size_t)n_win);
+    const Cmp packed{nfp,
+                     idx,
+                     nbr,
+                     eq6,
+                     reinterpret_cast<const uint32_t*>(tb + t_pos),
+                     reinterpret_cast<const uint2*>(tb + t_win),
+                     reinterpret_cast<const int2*>(tb + t_edge)};
+    const bool windows = windows_packable(b->q, n_win, nfp);
+    long long w0 = 0;
+    std::vector<CmpBlk> blk((size_t)(nfp / kBatchCmpAlign));
     // each instance's tables are built in the workspace's state buffers (free at this point), then
     // packed; compact_build checks the fluid count against the link words (and synchronises)
-    // padding nodes: bounce-back in every direction (their loads stay at their own index)
-    static_assert(kCmpBB == -1, "padding codes are written as all-ones bytes");
-    if (nfp > 0 && cudaMemsetAsync(nbr, 0xFF, sizeof(int32_t) * (size_t)(b->q - 1) * (size_t)nfp, s) != cudaSuccess)
-        return LBM_ERR_CUDA;
+    {
+        const lbm_status st = bpack_start_cmp(b->q, nfp, packed, s);
+        if (st != LBM_OK) return st;
+    }
     unsigned char* scratch = ws + b->o_ping[0];
     const size_t cap = b->o_ckpt - b->o_ping[0];
     for (int i = 0; i < b->n; ++i) {
-        const BCmpInst& c = ci[(size_t)i];
+        BCmpInst& c = ci[(size_t)i];
         PlanInfo I = b->info[(size_t)i];
         I.geo.link = b->insts[(size_t)i].g.link;
         if (compact_table_bytes(I, c.nf) > cap) return LBM_ERR_INVALID_ARG;
         Cmp local{0, nullptr, nullptr};
         const int32_t* cmap = nullptr;
-        lbm_status st = compact_build(I, c.nf, scratch, &local, &cmap, nullptr, s);
+        BCmpInst one = {};
+        lbm_status st = compact_build(I, c.nf, scratch, &local, &cmap, nullptr, &one, s);
         if (st != LBM_OK) return st;
-        st = bpack_launch_cmp(local, b->q, c.k0, nfp, idx, nbr, s);
+        c.n_int = windows ? one.n_int : 0;
+        c.lat = one.lat;
+        c.lat.inst = i;
+        const long long nw = window_count(I);
+        st = bpack_launch_cmp(local, b->q, c.k0, nfp, nw, w0, windows, packed, s);
         if (st != LBM_OK) return st;
+        w0 += nw;
         for (long long bl = c.k0 / kBatchCmpAlign; bl < (c.k0 + c.nf + kBatchCmpAlign - 1) / kBatchCmpAlign; ++bl)
-            blk[(size_t)bl] = i;
+            blk[(size_t)bl] = c.lat;
     }
     {
         const lbm_status st = eq6_bits_launch_cmp(b->q, nbr, nfp, eq6, s);  // padding nodes: bounce-back, bit 0
         if (st != LBM_OK) return st;
     }
+    // the same entries by class: blocks with boundary or padding nodes, then those of interior nodes alone
+    const size_t n_blk = blk.size();
+    unsigned n_mixed = 0;
+    for (int pass = 0; pass < 2; ++pass)
+        for (size_t bl = 0; bl < n_blk; ++bl) {
+            CmpBlk e = blk[bl];
+            const BCmpInst& c = ci[(size_t)e.inst];
+            const bool inside = (long long)(bl + 1) * kBatchCmpAlign <= c.k0 + c.n_int;
+            if (inside != (pass == 1)) continue;
+            e.pad = (int)bl;
+            blk.push_back(e);
+            n_mixed += pass == 0 ? 1 : 0;
+        }
     if (cudaMemcpyAsync(tb + t_insts, ci.data(), sizeof(BCmpInst) * ci.size(), cudaMemcpyHostToDevice, s) !=
             cudaSuccess ||
         (!blk.empty() &&
-         cudaMemcpyAsync(tb + t_blk, blk.data(), sizeof(int) * blk.size(), cudaMemcpyHostToDevice, s) != cudaSuccess))
+         cudaMemcpyAsync(tb + t_blk, blk.data(), sizeof(CmpBlk) * blk.size(), cudaMemcpyHostToDevice, s) != cudaSuccess))
         return LBM_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return LBM_ERR_CUDA;  // host vectors outlive the copies
     b->cinsts = ci;
-    b->blk_inst = blk;
     b->nfp = nfp;
     b->cmp_state_bytes = (size_t)b->q * (size_t)nfp * (size_t)b->prec;
     BCmpArgs& a = b->ca;
-    a.c = Cmp{nfp, idx, nbr, eq6};
+    a.c = packed;
     a.insts = reinterpret_cast<const BCmpInst*>(tb + t_insts);
-    a.blk_inst = reinterpret_cast<const int*>(tb + t_blk);
+    a.blks = reinterpret_cast<const CmpBlk*>(tb + t_blk);
+    a.blks_by_class = a.blks + nfp / kBatchCmpAlign;
+    a.n_mixed = n_mixed;
     a.n_blocks = (unsigned)(nfp / kBatchCmpAlign);
     a.q = b->q;
     a.prec = b->prec;

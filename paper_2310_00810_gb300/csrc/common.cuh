@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 
@@ -45,24 +46,27 @@ struct Bc {
     const double* rho_in;  // device: 1 or ny*nz entries
     short profile;         // 1: rho_in[z*ny + y], 0: rho_in[0]
     char uw_extrap = 0;    // 1: Eq. 6 takes u_w extrapolated to the pressure plane (LBM_ABB_U_EXTRAP)
-    char mrt = 0;          // 1: D2Q9 MRT collision (Eq. 16-18); its free rates are in the status section
-    char vel_inlet = 0;    // 1: velocity inlet through x = -1/2 (moving-wall bounce-back); u_in in the status section
+    char mrt = 0;          // 1: D2Q9 MRT collision (Eq. 16-18) with the free rates of mrt_rates
+    char vel_inlet = 0;    // 1: velocity inlet through x = -1/2 (moving-wall bounce-back) with u_in
     double rho_out;
     uint32_t* status;      // device status word (bounded waits latch LBM_ERR_TIMEOUT here)
     uint32_t wait_us = 2000000u;  // time bound of each mbarrier wait of the TMA kernels, in microseconds
     char test_stall = 0;   // 1: TMA producers issue no copies, so every consumer wait runs out (tests only)
     int t_level = 0;       // the time level this launch's streaming produces (f^t_level)
     int ramp_steps = 0;    // the velocity inlet starts gradually: u_in r(t_level), r = 1 from ramp_steps on
+    double ramp = 1.0;     // r(t_level), formed on the host (a device sine in FP64 costs the boundary warps microseconds)
+    double u_in[3] = {0.0, 0.0, 0.0};       // the velocity inlet's u_in
+    double mrt_rates[3] = {0.0, 0.0, 0.0};  // s_e, s_eps, s_q
     void* side_u = nullptr;  // in-place forward steps: the Eq. 6 nodes' velocities (read, then rewritten)
 };
 
 // The gradual start of the velocity inlet: r(t) = sin^2(pi t / (2 R)) for
 // 0 < t < R, 0 at t <= 0 and 1 from R on (R <= 0: no ramp).
-__device__ __forceinline__ double inlet_ramp(const Bc& bc)
+inline double inlet_ramp(int ramp_steps, int t)
 {
-    if (bc.ramp_steps <= 0 || bc.t_level >= bc.ramp_steps) return 1.0;
-    if (bc.t_level <= 0) return 0.0;
-    const double s = sin(3.14159265358979323846 * (double)bc.t_level / (2.0 * (double)bc.ramp_steps));
+    if (ramp_steps <= 0 || t >= ramp_steps) return 1.0;
+    if (t <= 0) return 0.0;
+    const double s = std::sin(3.14159265358979323846 * (double)t / (2.0 * (double)ramp_steps));
     return s * s;
 }
 
@@ -71,6 +75,7 @@ inline Bc at_time(const Bc& bc, int t)
 {
     Bc b = bc;
     b.t_level = t;
+    b.ramp = inlet_ramp(bc.ramp_steps, t);
     return b;
 }
 
@@ -82,6 +87,18 @@ struct Cmp {
     const int32_t* idx;    // idx[k]: dense node index of compact node k (interior nodes, then x = 0 / nx - 1)
     const int32_t* nbr;    // nbr[(i - 1) * nf + k], i = 1..Q-1: compact index of x - c_i, or kCmpBB / kCmpABB
     const uint32_t* eq6;   // bit k & 31 of eq6[k >> 5]: node k has an Eq. 6 / velocity-inlet link
+    const uint32_t* pos;   // pos[k]: window and column of interior node k (compact.cu)
+    const uint2* win;      // {fluid bits, compact index before them} of 30 columns of a row
+    const int2* edge;      // compact indices of the x = 0 / nx - 1 nodes of a window's row
+};
+constexpr int kWinCols = 30;  // columns per window (their bits and one to either side fill 32)
+
+// What a node's update needs to know about its lattice: a batch has one of
+// these per kBatchCmpAlign nodes.
+struct alignas(16) CmpBlk {
+    int inst;            // instance
+    int w_row, w_plane;  // windows per row and per plane
+    int pad;             // a batch's list of blocks by class: the block's number
 };
 
 struct BCmpInst;
@@ -123,6 +140,8 @@ struct PlanInfo {
     int tma_min_tiles;  // smallest tile count for which the TMA kernels are used
     size_t state_bytes;   // bytes of one internal state (Q N, or Q nf in the compact layout)
     Cmp cmp;
+    CmpBlk cmp_lat;          // how its kernels find neighbours
+    int cmp_int;             // interior nodes (the boundary columns follow)
     const int32_t* cmp_map;  // cmap[n]: compact index of dense node n, or -1 for a solid node (compact layout)
     const BCmpInst* cmp_inst;  // the lattice as a one-instance pack (compact layout; device)
 };
@@ -154,21 +173,6 @@ constexpr size_t kBarOffset = 64;  // byte offset of the PersistBar in the statu
 constexpr size_t kScalarCount = 8;    // double: ROI fluid-node count
 constexpr size_t kScalarWeight = 16;  // double: loss weight
 constexpr size_t kScalarTmp = 24;     // double: scratch
-constexpr size_t kMrtRates = 128;     // double[3]: s_e, s_eps, s_q of the MRT collision (written per call)
-constexpr size_t kInletVelocity = 160;  // double[3]: the velocity inlet's u_in (written per call)
-
-// The velocity inlet's u_in a kernel reads (Bc::vel_inlet).
-__device__ __forceinline__ const double* inlet_velocity(const uint32_t* status)
-{
-    return reinterpret_cast<const double*>(reinterpret_cast<const unsigned char*>(status) + kInletVelocity);
-}
-
-// The MRT rates a kernel reads (Bc::mrt): s_e, s_eps, s_q.
-__device__ __forceinline__ const double* mrt_rates(const uint32_t* status)
-{
-    return reinterpret_cast<const double*>(reinterpret_cast<const unsigned char*>(status) + kMrtRates);
-}
-
 // --------------------------------------------------------------- reductions
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -281,7 +285,7 @@ size_t compact_table_bytes(const PlanInfo& p, long long nf);
 // Batches in the fluid-only layout: the fluid nodes of every instance packed
 // into one compact state [Q][nfp], instance i at compact indices
 // [k0, k0 + nf), k0 a multiple of kBatchCmpAlign, so that every thread block
-// of the compact kernels belongs to one instance (blk_inst[block]).
+// of the compact kernels belongs to one instance (blks[block]).
 constexpr int kBatchCmpAlign = 256;
 struct BCmpInst {
     Geo g;              // the instance's sizes (the compact kernels use no link words)
@@ -289,12 +293,18 @@ struct BCmpInst {
     long long f_off;    // its dense [Q][N] arrays in a packed dense state (elements)
     long long in_off;   // inlet densities and their gradients
     long long acc_off;  // per-inlet-node accumulators (ny * nz)
-    int n_in, pad;
+    int n_in;
+    int n_int;          // interior nodes addressed through the windows
+    CmpBlk lat;
 };
 struct BCmpArgs {
     Cmp c;                   // c.nf = nfp (the packed stride), c.idx local dense indices, c.nbr packed codes
     const BCmpInst* insts;   // device
-    const int* blk_inst;     // device: instance of each kBatchCmpAlign-node block
+    const CmpBlk* blks;      // device: a batch's entry of each kBatchCmpAlign-node block
+    const CmpBlk* blks_by_class;  // device: the same entries, blocks with boundary or padding nodes first
+    unsigned n_mixed;        // how many of those
+    CmpBlk lat;              // a single lattice's entry
+    unsigned n_int;          // its interior nodes
     unsigned n_blocks;       // nfp / kBatchCmpAlign
     int q, prec, pdl;
     uint32_t* status;
@@ -305,12 +315,17 @@ lbm_status badjoint_launch_cmp(const BCmpArgs& a, int t0, const void* gprev, con
                                const double* rho_in, const double* tau, double rho_out, double* grad_acc,
                                double* partial, cudaStream_t s);
 lbm_status bgather_launch_cmp(const BCmpArgs& a, const void* dense, void* compact, cudaStream_t s);
-lbm_status bpack_launch_cmp(const Cmp& local, int q, long long k0, long long nfp, int32_t* idx, int32_t* nbr,
-                            cudaStream_t s);
+lbm_status bpack_launch_cmp(const Cmp& local, int q, long long k0, long long nfp, long long n_win, long long w0,
+                            bool windows, const Cmp& packed, cudaStream_t s);
+lbm_status bpack_start_cmp(int q, long long nfp, const Cmp& packed, cudaStream_t s);
+// whether a packed batch can use the windows (else every node goes through the table)
+bool windows_packable(int q, long long n_win, long long nfp);
+// windows of a lattice's rows, with one solid row (and plane) of padding on each side; 0: too many to address
+long long window_count(const PlanInfo& p);
 // the per-node Eq. 6 bit array of a (packed) table: bit k & 31 of bits[k >> 5]
 lbm_status eq6_bits_launch_cmp(int q, const int32_t* nbr, long long nf, uint32_t* bits, cudaStream_t s);
 lbm_status compact_build(const PlanInfo& p, long long nf, void* tables, Cmp* out, const int32_t** cmap_out,
-                         const BCmpInst** inst_out, cudaStream_t s);
+                         const BCmpInst** inst_out, BCmpInst* inst_host, cudaStream_t s);
 // Layouts of a fluid-only state (compact.cu): natural, or swapped (the
 // in-place schedule's layout of g^t and lambda^t at odd t).
 constexpr int kLayoutNatural = 0;
