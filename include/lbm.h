@@ -274,6 +274,21 @@ LBM_API lbm_status lbm_bind_geometry(lbm_plan* plan, const uint32_t* d_link);
 LBM_API lbm_status lbm_compact_size(const lbm_plan* plan, int64_t n_fluid, size_t* bytes);
 LBM_API lbm_status lbm_compact_bind(lbm_plan* plan, int64_t n_fluid, void* d_tables, void* stream);
 
+/* How the fluid-only layout's D2Q9 FP32 kernels round:
+ *   LBM_ROUND_NATIVE  the collision's last product and subtraction separately,
+ *                     and the terms of dL/dtau from f^eq - f summed without
+ *                     the equilibrium's 1 (default)
+ *   LBM_ROUND_DENSE   as the dense layout's TMA and register kernels: that
+ *                     product and subtraction as one fused operation, and the
+ *                     terms of dL/dtau from P = 1 + 3 c.u + ..., so that a
+ *                     lattice's results do not depend on which of the two
+ *                     layouts an automatic choice gives it
+ * With LBM_ABB_U_EXTRAP the dense layout has neither kernel and the setting has
+ * no effect.  Cached CUDA graphs are dropped on a change.  Errors: INVALID_ARG
+ * for an unknown mode. */
+enum { LBM_ROUND_NATIVE = 0, LBM_ROUND_DENSE = 1 };
+LBM_API lbm_status lbm_set_rounding(lbm_plan* plan, int32_t mode);
+
 /* T steps from rest (f = w_i, rho = 1: init_field of section 2.2), keeping
  * the checkpoints the adjoint needs in d_ws.
  *  d_rho_in  double[1 or ny nz]  inlet density (Eq. 6 rho_w at x = -1/2)

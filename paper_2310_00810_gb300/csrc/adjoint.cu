@@ -27,116 +27,86 @@
 
 namespace lbm {
 
-template <int Q, typename T, bool T0>
+// One node per thread; what a sweep does not change is read before the wait
+// for the preceding launch, and every load of f^t and lambda is issued
+// unconditionally from a selected address (k_step).  DENSE_ROUND: the rounding of
+// the dL/domega terms (adjoint_collision).
+template <int Q, typename T, bool T0, bool DENSE_ROUND>
 __global__ void __launch_bounds__(kStepThreads)
-    k_adjoint(const T* __restrict__ gprev, const T* __restrict__ lam_in, T* __restrict__ lam_out, Geo g, Bc bc,
-              const double* __restrict__ tau, double* __restrict__ grad_acc, double* __restrict__ partial)
+    k_adjoint(const T* gprev, const T* lam_in, T* lam_out, Geo g, Bc bc, const double* __restrict__ tau,
+              double* __restrict__ grad_acc, double* __restrict__ partial)
 {
-    pdl_enter();
     using L = Lattice<Q>;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
     const long long N = g.N, plane = (long long)g.nx * g.ny;
     const long long n = ((long long)z * g.ny + y) * g.nx + x;
-    uint32_t lw = kLinkSolid;
-    if (x < g.nx) lw = g.link[n];
-    double dom = 0.0;
-    if (!(lw & kLinkSolid)) {
-        // 1. f^t(x)
-        T f[Q];
+    const bool live = x < g.nx;
+    const uint32_t lw = live ? __ldg(g.link + n) : kLinkSolid;
+    const bool fluid = !(lw & kLinkSolid), xin = x == 0, xout = x == g.nx - 1;
+    const double rw = fluid && (xin || xout) ? wall_density(bc, g, xin, y, z) : 1.0;
+    const T omega = T(1) / T(*tau);
+    pdl_enter();
+    T dom = T(0);
+    T lamv[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) lamv[i] = T(0);
+    if (fluid) {
+        // 1. f^t(x), and 2. the transpose of streaming
+        T f[Q], mu[Q];
         if (T0) {
 #pragma unroll
             for (int i = 0; i < Q; ++i) f[i] = T(0);
         } else {
-            pull<Q, T>(f, gprev, n, x, y, z, lw, g, bc);
+            pull<Q, T>(f, gprev, n, x, lw, g, bc, rw);
+        }
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+            const int o = L::opp(j), cx = L::c(j, 0);
+            const bool own = ((lw >> o) & 1u) || (cx == -1 && xin) || (cx == 1 && xout);
+            const T* p = own ? lam_in + (long long)o * N : lam_in + (long long)j * N + link_offset<Q>(j, g.nx, plane);
+            mu[j] = p[n];
         }
         T drho, rho, u[3];
         moments<Q, T>(f, drho, rho, u);
-        const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        const T omega = T(1.0 / *tau);
-
-        // 2. transpose of streaming and boundaries
-        const bool xin = x == 0, xout = x == g.nx - 1;
-        T mu[Q];
         T G[3] = {T(0), T(0), T(0)};
-        double grw = 0.0;
-        T rwT = T(0);
-        if (xin || xout) rwT = T(xin ? (bc.profile ? bc.rho_in[(long long)z * g.ny + y] : bc.rho_in[0]) : bc.rho_out);
-        if (!(xin || xout)) {
-            // interior node: select the address, then load (all Q loads in flight together)
-#pragma unroll
-            for (int j = 0; j < Q; ++j) {
-                const int o = L::opp(j);
-                const bool bb = (lw >> o) & 1u;
-                mu[j] = lam_in[bb ? (long long)o * N + n : (long long)j * N + n + link_offset<Q>(j, g.nx, plane)];
-            }
-        } else {
+        if (xin || xout) {
+            const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+            const T rwT = T(rw);
+            double grw = 0.0;
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
                 const int o = L::opp(j), cx = L::c(j, 0);
-                if ((lw >> o) & 1u) {
-                    mu[j] = lam_in[(long long)o * N + n];
-                } else if ((cx == -1 && xin) || (cx == 1 && xout)) {
-                    const T li = lam_in[(long long)o * N + n];
-                    mu[j] = -li;
-                    const T cu = cdot<Q, T>(o, u);
-                    const T two_w = T(2.0 * L::w(o));
-                    if (xin) grw += (double)(li * two_w * (T(1) + T(4.5) * cu * cu - T(1.5) * uu));
-#pragma unroll
-                    for (int a = 0; a < L::D; ++a)
-                        G[a] += li * two_w * rwT * (T(9) * cu * T(L::c(o, a)) - T(3) * u[a]);
-                } else {
-                    mu[j] = lam_in[(long long)j * N + n + link_offset<Q>(j, g.nx, plane)];
-                }
-            }
-        }
-
-        // 3. transpose of the collision (BGK here, MRT in adjoint_collision_mrt)
-        T lamv[Q], domT = 0;
-        bool mrt_done = false;
-        if constexpr (Q == 9) {
-            if (bc.mrt) {
-                domT = adjoint_collision_mrt<T>(f, mu, drho, rho, u, G, omega, bc.mrt_rates, lamv);
-                mrt_done = true;
-            }
-        }
-        if (!mrt_done) {
-            T A = 0, B[3] = {T(0), T(0), T(0)};
-#pragma unroll
-            for (int j = 0; j < Q; ++j) {
-                const T cu = cdot<Q, T>(j, u);
-                const T wj = T(L::w(j));
-                const T P = T(1) + T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu;
-                const T feq = wj * (drho + rho * (T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu));
-                domT += mu[j] * (feq - f[j]);
-                A += mu[j] * wj * P;
+                if (((lw >> o) & 1u) || !((cx == -1 && xin) || (cx == 1 && xout))) continue;
+                const T li = mu[j];
+                mu[j] = -li;
+                const T cu = cdot<Q, T>(o, u);
+                const T two_w = T(2.0 * L::w(o));
+                if (xin) grw += (double)(li * two_w * (T(1) + T(4.5) * cu * cu - T(1.5) * uu));
 #pragma unroll
                 for (int a = 0; a < L::D; ++a)
-                    B[a] += mu[j] * wj * rho * (T(3 * L::c(j, a)) + T(9) * cu * T(L::c(j, a)) - T(3) * u[a]);
+                    G[a] += li * two_w * rwT * (T(9) * cu * T(L::c(o, a)) - T(3) * u[a]);
             }
-            const T inv = T(1) / rho;
-            T Bt[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) Bt[a] = (omega * B[a] + G[a]) * inv;
-            const T base = omega * A;
-            const T keep = T(1) - omega;
-#pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                T sk = keep * mu[k] + base;
-#pragma unroll
-                for (int a = 0; a < L::D; ++a) sk += Bt[a] * (T(L::c(k, a)) - u[a]);
-                lamv[k] = sk;
-            }
+            // 4. inlet gradient: one owner and one addition per launch, which nothing waits for
+            if (xin) atomicAdd(grad_acc + (long long)z * g.ny + y, grw);
         }
+        // 3. transpose of the collision
+        dom = adjoint_collision<Q, T, DENSE_ROUND>(f, mu, drho, rho, u, G, omega, lamv, bc);
+    }
+    if (stores_node(fluid, live, g, sizeof(T) == 4))
 #pragma unroll
         for (int k = 0; k < Q; ++k) lam_out[(long long)k * N + n] = lamv[k];
-
-        // 4. parameter gradients
-        dom = (double)domT;
-        if (xin) grad_acc[(long long)z * g.ny + y] += grw;
+    // dL/domega: warp sums in T (FP64 is slow on this part), the block's in FP64
+    __shared__ double s_part[kStepThreads / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dom += __shfl_xor_sync(0xffffffffu, dom, o);
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = (double)dom;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double bs = 0.0;
+#pragma unroll
+        for (int w = 0; w < kStepThreads / 32; ++w) bs += s_part[w];
+        atomicAdd(partial + ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, bs);
     }
-    const int tid = threadIdx.x;
-    const double bs = block_sum(dom, tid, blockDim.x);
-    if (tid == 0) partial[((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] += bs;
 }
 
 // Reverse of the extrapolated Eq. 6 velocity (Bc::uw_extrap), run after the
@@ -164,8 +134,8 @@ __global__ void __launch_bounds__(kStepThreads)
         const uint32_t lb = g.link[nb];
         if ((lb & kLinkSolid) || ((lb >> inward_dir<Q>(xin)) & 1u)) continue;
         T fb[Q], fe[Q], li[Q];
-        pull<Q, T>(fb, gprev, nb, xb, y, z, lb, g, bc);
-        pull<Q, T>(fe, gprev, ne, xe, y, z, g.link[ne], g, bc);
+        pull<Q, T>(fb, gprev, nb, xb, lb, g, bc, wall_density(bc, g, xin, y, z));
+        pull<Q, T>(fe, gprev, ne, xe, g.link[ne], g, bc, wall_density(bc, g, xe == 0, y, z));
         uint32_t eq6 = 0;
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
@@ -196,7 +166,7 @@ static void launch_uw(const PlanInfo& p, const void* gprev, const void* lam_in, 
              grad_acc);
 }
 
-template <int Q, typename T>
+template <int Q, typename T, bool DENSE_ROUND = false>
 static void launch(const PlanInfo& p, int t0, const void* gprev, const void* lam_in, void* lam_out, const Bc& bc,
                    const double* tau, double* grad_acc, double* partial, cudaStream_t s)
 {
@@ -204,9 +174,9 @@ static void launch(const PlanInfo& p, int t0, const void* gprev, const void* lam
     const T* li = static_cast<const T*>(lam_in);
     T* lo = static_cast<T*>(lam_out);
     if (t0)
-        launch_k(p.pdl, k_adjoint<Q, T, true>, dim3(p.grid), dim3(kStepThreads), 0, s, gp, li, lo, p.geo, bc, tau, grad_acc, partial);
+        launch_k(p.pdl, k_adjoint<Q, T, true, DENSE_ROUND>, dim3(p.grid), dim3(kStepThreads), 0, s, gp, li, lo, p.geo, bc, tau, grad_acc, partial);
     else
-        launch_k(p.pdl, k_adjoint<Q, T, false>, dim3(p.grid), dim3(kStepThreads), 0, s, gp, li, lo, p.geo, bc, tau, grad_acc, partial);
+        launch_k(p.pdl, k_adjoint<Q, T, false, DENSE_ROUND>, dim3(p.grid), dim3(kStepThreads), 0, s, gp, li, lo, p.geo, bc, tau, grad_acc, partial);
 }
 
 lbm_status adjoint_launch(const PlanInfo& plan, int t_is_zero, const void* gprev, const void* lam_in, void* lam_out,
@@ -231,6 +201,10 @@ lbm_status adjoint_launch(const PlanInfo& plan, int t_is_zero, const void* gprev
             else if (p.prec == 4) launch_uw<19, float>(p, gprev, lam_in, lam_out, bc, grad_acc, s);
             else launch_uw<19, double>(p, gprev, lam_in, lam_out, bc, grad_acc, s);
         }
+        return cuda_status(cudaGetLastError());
+    }
+    if (auto_scalar(plan, plan.adj_family)) {
+        launch<9, float, true>(plan, t_is_zero, gprev, lam_in, lam_out, bc, tau, grad_acc, partial, s);
         return cuda_status(cudaGetLastError());
     }
     const PlanInfo p = with_family(plan, plan.adj_family);

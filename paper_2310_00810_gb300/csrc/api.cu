@@ -352,6 +352,7 @@ lbm_status lbm_plan_create(const lbm_desc* d, lbm_plan** out)
     const char* tmin = std::getenv("LBM_TMA_MIN_TILES");
     I.use_tma = I.max_vec >= 2 && !(tma && tma[0] == '0');
     I.tma_min_tiles = tmin ? std::atoi(tmin) : 1;
+    I.tma_named = tmin ? 1 : 0;
     const char* sv = std::getenv("LBM_STEP_VARIANT");
     I.step_variant = sv ? std::atoi(sv) : 0;
     const char* tv = std::getenv("LBM_TMA_VARIANT");
@@ -470,6 +471,14 @@ lbm_status lbm_set_collision(lbm_plan* p, int32_t mode, double s_e, double s_eps
         p->info.mrt_rates[2] = s_q;
     }
     p->info.mrt = mode == LBM_COLLISION_MRT ? 1 : 0;
+    drop_graphs(p);
+    return LBM_OK;
+}
+
+lbm_status lbm_set_rounding(lbm_plan* p, int32_t mode)
+{
+    if (!p || (mode != LBM_ROUND_NATIVE && mode != LBM_ROUND_DENSE)) return LBM_ERR_INVALID_ARG;
+    p->info.dense_round = mode == LBM_ROUND_DENSE ? 1 : 0;
     drop_graphs(p);
     return LBM_OK;
 }

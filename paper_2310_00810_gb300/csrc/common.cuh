@@ -129,6 +129,8 @@ struct PlanInfo {
     int aa;           // 1: in-place (AA-pattern) streaming in the fluid-only layout
     int uw_extrap;    // 1: Eq. 6 with the extrapolated wall velocity (one-node-per-thread or fluid-only kernels)
     int mrt;          // 1: D2Q9 MRT collision (one-node-per-thread or fluid-only kernels)
+    int dense_round;  // 1: LBM_ROUND_DENSE
+    int tma_named;    // 1: the environment sets from which size the TMA kernels are used
     int vel_inlet;    // 1: velocity inlet instead of Eq. 6 at x = -1/2 (fluid-only kernels)
     double u_in[3];   // its velocity
     int ramp_steps;   // its gradual start (0: none)
@@ -280,6 +282,17 @@ inline PlanInfo with_family(const PlanInfo& p, int family)
     return q;
 }
 
+// Whether an automatic choice of kernels runs the one-node-per-thread ones
+// where the TMA ones apply too: up to about half a million nodes, where a
+// launch is latency (a time step of a gradient evaluation, TMA and one node
+// per thread: 128x64 11.6 and 5.5 us, 512x256 13.3 and 10.5, 1024x512 33.4 and
+// 27.3; 2048x1024 103 and 110).
+inline bool auto_scalar(const PlanInfo& p, int family)
+{
+    return family == LBM_FAMILY_AUTO && p.q == 9 && p.prec == 4 && p.use_tma && !p.tma_named && p.geo.nx % 2 == 0 &&
+           p.geo.N <= 600000;
+}
+
 size_t compact_table_bytes(const PlanInfo& p, long long nf);
 
 // Batches in the fluid-only layout: the fluid nodes of every instance packed
@@ -305,6 +318,7 @@ struct BCmpArgs {
     unsigned n_mixed;        // how many of those
     CmpBlk lat;              // a single lattice's entry
     unsigned n_int;          // its interior nodes
+    bool dense_round = false;  // LBM_ROUND_DENSE (D2Q9 FP32)
     unsigned n_blocks;       // nfp / kBatchCmpAlign
     int q, prec, pdl;
     uint32_t* status;

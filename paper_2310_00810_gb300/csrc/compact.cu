@@ -756,47 +756,6 @@ struct CmpOrder {
     __device__ __forceinline__ unsigned block(unsigned b) const { return b < first || rev ? n - 1 - b : b - first; }
 };
 
-// Transpose of the collision (adjoint.cu, step 3) at one node, from f^t (its
-// moments drho, rho, u) and mu = dL/df*: gives lambda^t and returns the
-// node's dL/domega term.  G holds the Eq. 6 velocity terms (zero inside).
-template <int Q, typename T>
-__device__ __forceinline__ T adjoint_collision(const T (&f)[Q], const T (&mu)[Q], T drho, T rho, const T (&u)[3],
-                                               const T (&G)[3], T omega, T (&lam)[Q], const Bc& bc)
-{
-    using L = Lattice<Q>;
-    if constexpr (Q == 9) {
-        if (bc.mrt) return adjoint_collision_mrt<T>(f, mu, drho, rho, u, G, omega, bc.mrt_rates, lam);
-    }
-    const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    T A = 0, B[3] = {T(0), T(0), T(0)}, domT = 0;
-#pragma unroll
-    for (int j = 0; j < Q; ++j) {
-        const T cu = cdot<Q, T>(j, u);
-        const T wj = T(L::w(j));
-        const T P = T(1) + T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu;
-        const T feq = wj * (drho + rho * (T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu));
-        domT += mu[j] * (feq - f[j]);
-        A += mu[j] * wj * P;
-#pragma unroll
-        for (int a = 0; a < L::D; ++a)
-            B[a] += mu[j] * wj * rho * (T(3 * L::c(j, a)) + T(9) * cu * T(L::c(j, a)) - T(3) * u[a]);
-    }
-    const T inv = T(1) / rho;
-    T Bt[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Bt[a] = (omega * B[a] + G[a]) * inv;
-    const T base = omega * A;
-    const T keep = T(1) - omega;
-#pragma unroll
-    for (int kk = 0; kk < Q; ++kk) {
-        T s = keep * mu[kk] + base;
-#pragma unroll
-        for (int a = 0; a < L::D; ++a) s += Bt[a] * (T(L::c(kk, a)) - u[a]);
-        lam[kk] = s;
-    }
-    return domT;
-}
-
 // Adjoint step in the compact layout: the gather form of adjoint.cu.  The
 // forward copies f*_j(x) to x + c_j, the node that pulls direction j from x;
 // its compact index is the code of direction opp(j) at x (x + c_j = x - c_opp(j)).
@@ -868,14 +827,14 @@ __device__ __forceinline__ void pull_adjoint_table(T (&f)[Q], T (&mu)[Q], T (&G)
 
 // lambda^t of a node from f^t, mu and G (the transpose of the collision),
 // stored; returns its dL/domega term.
-template <int Q, typename T, int OUT>
+template <int Q, typename T, int OUT, bool DENSE_ROUND>
 __device__ __forceinline__ T adjoint_node(const T (&f)[Q], const T (&mu)[Q], const T (&G)[3], T* lam_out,
                                           const Node& nd, const Cmp& c, const Bc& tmpl, T omega)
 {
     T drho, rho, u[3];
     moments<Q, T>(f, drho, rho, u);
     T lam[Q];
-    const T dom = adjoint_collision<Q, T>(f, mu, drho, rho, u, G, omega, lam, tmpl);
+    const T dom = adjoint_collision<Q, T, DENSE_ROUND>(f, mu, drho, rho, u, G, omega, lam, tmpl);
     if (OUT == kOutScatter) {  // lambda_m(x) to (x - c_m, opp(m)) where that node is fluid
         store_scattered<Q, T, -1>(lam_out, lam, nd, c);
     } else {
@@ -989,7 +948,7 @@ constexpr int kMinBlocks = sizeof(T) == 8 ? 2 : 4;
 // for the preceding launch, or (in place) hit a line that another block has
 // rewritten since.  Padding nodes of a batch are skipped: nothing ever reads
 // them.
-template <int Q, typename T, int MODE, bool DIN, int IN, int OUT>
+template <int Q, typename T, int MODE, bool DIN, int IN, int OUT, bool DENSE_ROUND>
 __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
     k_step_cmp(const T* src, T* dst, Cmp c, CmpBlk lat, const BCmpInst* __restrict__ insts,
                const CmpBlk* __restrict__ blks, Bc tmpl, const double* __restrict__ tau, CmpOrder ord)
@@ -1023,7 +982,7 @@ __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
         pdl_enter();
         pull_table<Q, T, IN, kInPlace<IN, OUT>>(v, src, k, wall, (size_t)c.nf, code, tmpl, I, side);
     }
-    if (MODE != kStreamOnly) collide_any<Q, T>(v, omega, tmpl);
+    if (MODE != kStreamOnly) collide_any<Q, T, DENSE_ROUND>(v, omega, tmpl);
     store_node<Q, T, OUT>(dst, v, nd, c, I);
     if (MODE != kStreamOnly && side && (MODE == kCollideOnly || nd.bnd()) && eq6_bit(c, k))
         keep_velocity<Q, T>(v, wall.sd, tmpl, I);
@@ -1108,7 +1067,7 @@ struct Ahead {
 };
 
 // One node of a block with boundary or padding nodes.
-template <int Q, typename T, bool BATCH>
+template <int Q, typename T, bool BATCH, bool DENSE_ROUND>
 __device__ __forceinline__ void pipe_step_node(const PipeArgs<T>& A, unsigned b)
 {
     Node nd;
@@ -1127,17 +1086,17 @@ __device__ __forceinline__ void pipe_step_node(const PipeArgs<T>& A, unsigned b)
         window_neighbours<Q>(nb, A.c, nd.blk, nd.k, nd.pos);
         pull_interior<Q, T, kInGather, false>(v, A.src, nd.k, (uint32_t)A.c.nf, nb);
     }
-    collide_any<Q, T>(v, T(1) / T(A.tau[nd.blk.inst]), A.tmpl);
+    collide_any<Q, T, DENSE_ROUND>(v, T(1) / T(A.tau[nd.blk.inst]), A.tmpl);
     store_node<Q, T, kOutOwn>(A.out, v, nd, A.c, I);
 }
 
-template <int Q, typename T, bool BATCH, int MINB>
+template <int Q, typename T, bool BATCH, bool DENSE_ROUND, int MINB>
 __global__ void __launch_bounds__(kPipeThreads, MINB) k_step_cmp_pipe(const __grid_constant__ PipeArgs<T> A)
 {
     unsigned b = blockIdx.x;
     if (b < A.ord.first) {
         pdl_enter();
-        for (; b < A.ord.first; b += gridDim.x) pipe_step_node<Q, T, BATCH>(A, b);
+        for (; b < A.ord.first; b += gridDim.x) pipe_step_node<Q, T, BATCH, DENSE_ROUND>(A, b);
         if (b >= A.ord.n) return;
     }
     Ahead<Q, T, BATCH> a;
@@ -1156,7 +1115,7 @@ __global__ void __launch_bounds__(kPipeThreads, MINB) k_step_cmp_pipe(const __gr
             cur = blk.inst;
             omega = T(1) / T(A.tau[cur]);
         }
-        collide_any<Q, T>(v, omega, A.tmpl);
+        collide_any<Q, T, DENSE_ROUND>(v, omega, A.tmpl);
         const int32_t k = a.node(blk);
 #pragma unroll
         for (int i = 0; i < Q; ++i) (A.out + (size_t)i * (size_t)A.c.nf)[k] = v[i];
@@ -1182,7 +1141,7 @@ __global__ void __launch_bounds__(kPipeThreads, MINB) k_step_cmp_pipe(const __gr
 }
 
 // One node of a block with boundary or padding nodes; every thread calls it.
-template <int Q, typename T, bool BATCH>
+template <int Q, typename T, bool BATCH, bool DENSE_ROUND>
 __device__ __forceinline__ void pipe_adjoint_node(const PipeArgs<T>& A, unsigned b)
 {
     Node nd;
@@ -1202,18 +1161,18 @@ __device__ __forceinline__ void pipe_adjoint_node(const PipeArgs<T>& A, unsigned
             window_neighbours<Q>(nb, A.c, nd.blk, nd.k, nd.pos);
             pull_adjoint<Q, T, false, kInGather, false>(f, mu, A.src, A.lam_in, nd.k, (uint32_t)A.c.nf, nb);
         }
-        dom = adjoint_node<Q, T, kOutOwn>(f, mu, G, A.out, nd, A.c, A.tmpl, T(1) / T(A.tau[nd.blk.inst]));
+        dom = adjoint_node<Q, T, kOutOwn, DENSE_ROUND>(f, mu, G, A.out, nd, A.c, A.tmpl, T(1) / T(A.tau[nd.blk.inst]));
     }
     add_warp_partial<T>(dom, nd.k < (int32_t)A.c.nf, nd.k, A.partial);
 }
 
-template <int Q, typename T, bool BATCH, int MINB>
+template <int Q, typename T, bool BATCH, bool DENSE_ROUND, int MINB>
 __global__ void __launch_bounds__(kPipeThreads, MINB) k_adjoint_cmp_pipe(const __grid_constant__ PipeArgs<T> A)
 {
     unsigned b = blockIdx.x;
     if (b < A.ord.first) {
         pdl_enter();
-        for (; b < A.ord.first; b += gridDim.x) pipe_adjoint_node<Q, T, BATCH>(A, b);
+        for (; b < A.ord.first; b += gridDim.x) pipe_adjoint_node<Q, T, BATCH, DENSE_ROUND>(A, b);
         if (b >= A.ord.n) return;
     }
     Ahead<Q, T, BATCH> a;
@@ -1235,7 +1194,7 @@ __global__ void __launch_bounds__(kPipeThreads, MINB) k_adjoint_cmp_pipe(const _
         const T G[3] = {T(0), T(0), T(0)};
         Node nd;
         nd.k = a.node(blk);
-        const T dom = adjoint_node<Q, T, kOutOwn>(f, mu, G, A.out, nd, A.c, A.tmpl, omega);
+        const T dom = adjoint_node<Q, T, kOutOwn, DENSE_ROUND>(f, mu, G, A.out, nd, A.c, A.tmpl, omega);
         add_warp_partial<T>(dom, true, nd.k, A.partial);
     };
     T f0[Q], m0[Q], f1[Q], m1[Q];
@@ -1262,7 +1221,7 @@ __global__ void __launch_bounds__(kPipeThreads, MINB) k_adjoint_cmp_pipe(const _
 // [k0 / 32, (k0 + nf + 31) / 32).  lam_in == lam_out is allowed for the
 // in-place pairs (as for k_step_cmp: disjoint slot sets, all loads of a node
 // before its stores).
-template <int Q, typename T, bool T0, int IN, int OUT>
+template <int Q, typename T, bool T0, int IN, int OUT, bool DENSE_ROUND>
 __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
     k_adjoint_cmp(const T* gprev, const T* lam_in, T* lam_out, Cmp c, CmpBlk lat,
                   const BCmpInst* __restrict__ insts, const CmpBlk* __restrict__ blks, Bc tmpl,
@@ -1294,7 +1253,7 @@ __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
         pdl_enter();
     }
     T dom = T(0);
-    if (nd.live()) dom = adjoint_node<Q, T, OUT>(f, mu, G, lam_out, nd, c, tmpl, omega);
+    if (nd.live()) dom = adjoint_node<Q, T, OUT, DENSE_ROUND>(f, mu, G, lam_out, nd, c, tmpl, omega);
     add_warp_partial<T>(dom, k < (int32_t)c.nf, k, partial);
 }
 
@@ -1362,6 +1321,7 @@ BCmpArgs single_args(const PlanInfo& p, uint32_t* status)
     a.insts = p.cmp_inst;
     a.blks = nullptr;
     a.lat = p.cmp_lat;
+    a.dense_round = p.dense_round && !p.uw_extrap;
     a.n_int = (unsigned)p.cmp_int;
     a.n_blocks = cmp_grid(p.cmp.nf);
     a.q = p.q;
@@ -1421,8 +1381,8 @@ CmpOrder pipe_order(const BCmpArgs& a, int t)
     return o;
 }
 
-template <int Q, typename T>
-void launch_step(const BCmpArgs& a, int mode, const void* src, void* dst, bool din, bool dout, int lin, int lout,
+template <int Q, typename T, bool DENSE_ROUND>
+void launch_step_as(const BCmpArgs& a, int mode, const void* src, void* dst, bool din, bool dout, int lin, int lout,
                  const Bc& tmpl, const double* tau, cudaStream_t s)
 {
     const T* x = static_cast<const T*>(src);
@@ -1436,7 +1396,7 @@ void launch_step(const BCmpArgs& a, int mode, const void* src, void* dst, bool d
     };
     if (mode == kStreamCollide) {
         if (swap_in) {  // the local step: its interior nodes read their own slots
-            go(k_step_cmp<Q, T, kStreamCollide, false, kInLocal, kOutOwn>, grid);
+            go(k_step_cmp<Q, T, kStreamCollide, false, kInLocal, kOutOwn, DENSE_ROUND>, grid);
             return;
         }
         if constexpr (kPipe<Q, T>) {
@@ -1444,27 +1404,40 @@ void launch_step(const BCmpArgs& a, int mode, const void* src, void* dst, bool d
                 constexpr int MINB = 5;
                 const PipeArgs<T> A{x, nullptr, y, a.c, a.lat, a.insts, a.blks_by_class, tmpl, tau, nullptr, nullptr,
                                     pipe_order(a, tmpl.t_level)};
-                if (a.blks) launch_pipe(a.pdl, k_step_cmp_pipe<Q, T, true, MINB>, A, s);
-                else launch_pipe(a.pdl, k_step_cmp_pipe<Q, T, false, MINB>, A, s);
+                if (a.blks) launch_pipe(a.pdl, k_step_cmp_pipe<Q, T, true, DENSE_ROUND, MINB>, A, s);
+                else launch_pipe(a.pdl, k_step_cmp_pipe<Q, T, false, DENSE_ROUND, MINB>, A, s);
                 return;
             }
         }
-        if (swap_out) go(k_step_cmp<Q, T, kStreamCollide, false, kInGather, kOutScatter>, grid);
-        else go(k_step_cmp<Q, T, kStreamCollide, false, kInGather, kOutOwn>, grid);
+        if (swap_out) go(k_step_cmp<Q, T, kStreamCollide, false, kInGather, kOutScatter, DENSE_ROUND>, grid);
+        else go(k_step_cmp<Q, T, kStreamCollide, false, kInGather, kOutOwn, DENSE_ROUND>, grid);
     } else if (mode == kCollideOnly && din) {
-        go(k_step_cmp<Q, T, kCollideOnly, true, kInGather, kOutOwn>, grid);
+        go(k_step_cmp<Q, T, kCollideOnly, true, kInGather, kOutOwn, DENSE_ROUND>, grid);
     } else if (mode == kCollideOnly) {
-        go(k_step_cmp<Q, T, kCollideOnly, false, kInGather, kOutOwn>, grid);
+        go(k_step_cmp<Q, T, kCollideOnly, false, kInGather, kOutOwn, DENSE_ROUND>, grid);
     } else if (dout && swap_in) {
-        go(k_step_cmp<Q, T, kStreamOnly, false, kInLocal, kOutDense>, grid);
+        go(k_step_cmp<Q, T, kStreamOnly, false, kInLocal, kOutDense, DENSE_ROUND>, grid);
     } else if (dout) {
-        go(k_step_cmp<Q, T, kStreamOnly, false, kInGather, kOutDense>, grid);
+        go(k_step_cmp<Q, T, kStreamOnly, false, kInGather, kOutDense, DENSE_ROUND>, grid);
     } else {
-        go(k_step_cmp<Q, T, kStreamOnly, false, kInGather, kOutOwn>, grid);
+        go(k_step_cmp<Q, T, kStreamOnly, false, kInGather, kOutOwn, DENSE_ROUND>, grid);
     }
 }
 
-template <int Q, typename T, int IN, int OUT>
+template <int Q, typename T>
+void launch_step(const BCmpArgs& a, int mode, const void* src, void* dst, bool din, bool dout, int lin, int lout,
+                 const Bc& tmpl, const double* tau, cudaStream_t s)
+{
+    if constexpr (Q == 9 && std::is_same<T, float>::value) {
+        if (a.dense_round && mode != kStreamOnly) {
+            launch_step_as<Q, T, true>(a, mode, src, dst, din, dout, lin, lout, tmpl, tau, s);
+            return;
+        }
+    }
+    launch_step_as<Q, T, false>(a, mode, src, dst, din, dout, lin, lout, tmpl, tau, s);
+}
+
+template <int Q, typename T, int IN, int OUT, bool DENSE_ROUND>
 void launch_adjoint_as(const BCmpArgs& a, int t0, const T* gp, const T* li, T* lo, const Bc& tmpl, const double* tau,
                        double* grad_acc, double* partial, cudaStream_t s)
 {
@@ -1479,13 +1452,13 @@ void launch_adjoint_as(const BCmpArgs& a, int t0, const T* gp, const T* li, T* l
             constexpr int MINB = 4;
             const PipeArgs<T> A{gp, li, lo, a.c, a.lat, a.insts, a.blks_by_class, tmpl, tau, grad_acc, partial,
                                 pipe_order(a, tmpl.t_level)};
-            if (a.blks) launch_pipe(a.pdl, k_adjoint_cmp_pipe<Q, T, true, MINB>, A, s);
-            else launch_pipe(a.pdl, k_adjoint_cmp_pipe<Q, T, false, MINB>, A, s);
+            if (a.blks) launch_pipe(a.pdl, k_adjoint_cmp_pipe<Q, T, true, DENSE_ROUND, MINB>, A, s);
+            else launch_pipe(a.pdl, k_adjoint_cmp_pipe<Q, T, false, DENSE_ROUND, MINB>, A, s);
             return;
         }
     }
-    if (t0) go(k_adjoint_cmp<Q, T, true, IN, OUT>);
-    else go(k_adjoint_cmp<Q, T, false, IN, OUT>);
+    if (t0) go(k_adjoint_cmp<Q, T, true, IN, OUT, DENSE_ROUND>);
+    else go(k_adjoint_cmp<Q, T, false, IN, OUT, DENSE_ROUND>);
 }
 
 // lin: the layout of g^{t-1} and lambda^{t+1} (the same in every sweep);
@@ -1497,12 +1470,22 @@ void launch_adjoint(const BCmpArgs& a, int t0, const void* gprev, const void* la
     const T* gp = static_cast<const T*>(gprev);
     const T* li = static_cast<const T*>(lam_in);
     T* lo = static_cast<T*>(lam_out);
-    if (lin == kLayoutSwapped)
-        launch_adjoint_as<Q, T, kInLocal, kOutOwn>(a, t0, gp, li, lo, tmpl, tau, grad_acc, partial, s);
-    else if (lout == kLayoutSwapped)
-        launch_adjoint_as<Q, T, kInGather, kOutScatter>(a, t0, gp, li, lo, tmpl, tau, grad_acc, partial, s);
-    else
-        launch_adjoint_as<Q, T, kInGather, kOutOwn>(a, t0, gp, li, lo, tmpl, tau, grad_acc, partial, s);
+    auto as = [&](auto round) {
+        constexpr bool DR = decltype(round)::value;
+        if (lin == kLayoutSwapped)
+            launch_adjoint_as<Q, T, kInLocal, kOutOwn, DR>(a, t0, gp, li, lo, tmpl, tau, grad_acc, partial, s);
+        else if (lout == kLayoutSwapped)
+            launch_adjoint_as<Q, T, kInGather, kOutScatter, DR>(a, t0, gp, li, lo, tmpl, tau, grad_acc, partial, s);
+        else
+            launch_adjoint_as<Q, T, kInGather, kOutOwn, DR>(a, t0, gp, li, lo, tmpl, tau, grad_acc, partial, s);
+    };
+    if constexpr (Q == 9 && std::is_same<T, float>::value) {
+        if (a.dense_round) {
+            as(std::true_type{});
+            return;
+        }
+    }
+    as(std::false_type{});
 }
 
 lbm_status step_any(const BCmpArgs& a, int mode, const void* src, void* dst, bool din, bool dout, const Bc& tmpl,

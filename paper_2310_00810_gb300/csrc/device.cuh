@@ -45,8 +45,11 @@ __device__ __forceinline__ T cdot(int i, const T (&u)[3])
     return s;
 }
 
-// BGK collision (Eq. 4-5) in place on shifted populations.
-template <int Q, typename T>
+// BGK collision (Eq. 4-5) in place on shifted populations.  FUSED: the last
+// product and subtraction as one rounding, which is what the compiler makes
+// of it in the vectorised and TMA kernels; where a kernel also holds the MRT
+// collision it rounds twice.
+template <int Q, typename T, bool FUSED = false>
 __device__ __forceinline__ void collide(T (&v)[Q], T omega)
 {
     using L = Lattice<Q>;
@@ -57,7 +60,7 @@ __device__ __forceinline__ void collide(T (&v)[Q], T omega)
     for (int i = 0; i < Q; ++i) {
         T cu = cdot<Q, T>(i, u);
         T feq = T(L::w(i)) * (drho + rho * (T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu));
-        v[i] = v[i] - omega * (v[i] - feq);
+        v[i] = FUSED ? fma(-omega, v[i] - feq, v[i]) : v[i] - omega * (v[i] - feq);
     }
 }
 
@@ -127,7 +130,7 @@ __device__ __forceinline__ void collide_mrt(T (&v)[9], T omega, const double (&r
 }
 
 // BGK (Eq. 4-5) or, on D2Q9 plans with Bc::mrt, MRT.
-template <int Q, typename T>
+template <int Q, typename T, bool FUSED = false>
 __device__ __forceinline__ void collide_any(T (&v)[Q], T omega, const Bc& bc)
 {
     if constexpr (Q == 9) {
@@ -136,7 +139,7 @@ __device__ __forceinline__ void collide_any(T (&v)[Q], T omega, const Bc& bc)
             return;
         }
     }
-    collide<Q, T>(v, omega);
+    collide<Q, T, FUSED>(v, omega);
 }
 
 // Transpose of the MRT collision at one node, from f^t (moments drho, rho, u)
@@ -276,14 +279,74 @@ __device__ __forceinline__ double adjoint_uw_delta(const T (&fb)[Q], const T (&f
     return dgrw;
 }
 
-// Pull with boundaries: fills v with what node n (at x, y, z) receives.
+// Transpose of the collision (adjoint.cu, step 3) at one node, from f^t (its
+// moments drho, rho, u) and mu = dL/df*: gives lambda^t and returns the
+// node's dL/domega term.  G holds the Eq. 6 velocity terms (zero inside).
+// DENSE_ROUND: f^eq in that term formed from P (as the vectorised and TMA
+// kernels round it) instead of P - 1 summed without its 1.
+template <int Q, typename T, bool DENSE_ROUND = false>
+__device__ __forceinline__ T adjoint_collision(const T (&f)[Q], const T (&mu)[Q], T drho, T rho, const T (&u)[3],
+                                               const T (&G)[3], T omega, T (&lam)[Q], const Bc& bc)
+{
+    using L = Lattice<Q>;
+    if constexpr (Q == 9) {
+        if (bc.mrt) return adjoint_collision_mrt<T>(f, mu, drho, rho, u, G, omega, bc.mrt_rates, lam);
+    }
+    const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    T A = 0, B[3] = {T(0), T(0), T(0)}, domT = 0;
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+        const T cu = cdot<Q, T>(j, u);
+        const T wj = T(L::w(j));
+        const T P = T(1) + T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu;
+        const T feq = wj * (drho + rho * (DENSE_ROUND ? P - T(1) : T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu));
+        domT += mu[j] * (feq - f[j]);
+        A += mu[j] * wj * P;
+#pragma unroll
+        for (int a = 0; a < L::D; ++a)
+            B[a] += mu[j] * wj * rho * (T(3 * L::c(j, a)) + T(9) * cu * T(L::c(j, a)) - T(3) * u[a]);
+    }
+    const T inv = T(1) / rho;
+    T Bt[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) Bt[a] = (omega * B[a] + G[a]) * inv;
+    const T base = omega * A;
+    const T keep = T(1) - omega;
+#pragma unroll
+    for (int kk = 0; kk < Q; ++kk) {
+        T s = keep * mu[kk] + base;
+#pragma unroll
+        for (int a = 0; a < L::D; ++a) s += Bt[a] * (T(L::c(kk, a)) - u[a]);
+        lam[kk] = s;
+    }
+    return domT;
+}
+
+// The wall density of Eq. 6 at a node of column 0 or nx - 1.
+__device__ __forceinline__ double wall_density(const Bc& bc, const Geo& g, bool xin, int y, int z)
+{
+    return xin ? (bc.profile ? bc.rho_in[(long long)z * g.ny + y] : bc.rho_in[0]) : bc.rho_out;
+}
+
+// Pull with boundaries: fills v with what node n (at column x) receives; rw
+// is its wall density where x = 0 or nx - 1.  Every address is selected and
+// then loaded unconditionally (a population that does not come from a
+// neighbour starts from the node's own one of the opposite direction), so
+// the loads issue together instead of one branch, and one wait, at a time.
 template <int Q, typename T>
-__device__ __forceinline__ void pull(T (&v)[Q], const T* __restrict__ src, long long n, int x, int y, int z,
-                                     uint32_t lw, const Geo& g, const Bc& bc)
+__device__ __forceinline__ void pull(T (&v)[Q], const T* src, long long n, int x, uint32_t lw, const Geo& g,
+                                     const Bc& bc, double rw)
 {
     using L = Lattice<Q>;
     const long long N = g.N, plane = (long long)g.nx * g.ny;
     const bool xin = x == 0, xout = x == g.nx - 1;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const int cx = L::c(i, 0);
+        const bool own = ((lw >> i) & 1u) || (cx == 1 && xin) || (cx == -1 && xout);
+        const T* p = own ? src + (long long)L::opp(i) * N : src + (long long)i * N - link_offset<Q>(i, g.nx, plane);
+        v[i] = p[n];
+    }
     if (xin || xout) {
         // the node's own velocity u(x, t) for Eq. 6, from its local state
         T loc[Q];
@@ -294,30 +357,27 @@ __device__ __forceinline__ void pull(T (&v)[Q], const T* __restrict__ src, long 
         if (bc.uw_extrap && !((lw >> inward_dir<Q>(xin)) & 1u))
             extrapolate_wall_velocity<Q, T>(u, src, N, xin ? n + 1 : n - 1);
         const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        const double rw = xin ? (bc.profile ? bc.rho_in[(long long)z * g.ny + y] : bc.rho_in[0]) : bc.rho_out;
         const T drw = T(rw - 1.0), rwT = T(rw);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const int cx = L::c(i, 0);
-            if ((lw >> i) & 1u) {
-                v[i] = loc[L::opp(i)];
-            } else if ((cx == 1 && xin) || (cx == -1 && xout)) {
+            if (!((lw >> i) & 1u) && ((cx == 1 && xin) || (cx == -1 && xout))) {
                 const T cu = cdot<Q, T>(i, u);
-                v[i] = -loc[L::opp(i)] + T(2.0 * L::w(i)) * (drw + rwT * (T(4.5) * cu * cu - T(1.5) * uu));
-            } else {
-                v[i] = src[(long long)i * N + n - link_offset<Q>(i, g.nx, plane)];
+                v[i] = -v[i] + T(2.0 * L::w(i)) * (drw + rwT * (T(4.5) * cu * cu - T(1.5) * uu));
             }
         }
-    } else {
-        // the address is selected, then loaded unconditionally: the Q loads
-        // then issue together instead of one branch (and one wait) at a time
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const bool bb = (lw >> i) & 1u;
-            const long long a = bb ? (long long)L::opp(i) * N + n : (long long)i * N + n - link_offset<Q>(i, g.nx, plane);
-            v[i] = src[a];
-        }
     }
+}
+
+// Whether a lane stores its node: fluid nodes, and the solid ones (as zeros)
+// of every 32-byte sector that holds a fluid node, so that DRAM never has to
+// merge a partly written sector.  Called by whole warps.
+__device__ __forceinline__ bool stores_node(bool fluid, bool live, const Geo& g, bool fp32)
+{
+    const unsigned m = __ballot_sync(0xffffffffu, fluid);
+    if (!live) return false;
+    const int lane = (int)(threadIdx.x & 31u);
+    return !g.skip_sectors || ((m >> (fp32 ? lane & 24 : lane & 28)) & (fp32 ? 0xffu : 0xfu)) != 0u;
 }
 
 }  // namespace lbm

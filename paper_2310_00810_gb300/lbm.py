@@ -29,11 +29,12 @@ LBM_LINK_SOLID = 0x80000000
 LBM_FAMILY_AUTO, LBM_FAMILY_SCALAR, LBM_FAMILY_VEC, LBM_FAMILY_TMA = 0, 1, 2, 3
 LBM_ABB_U_NODE, LBM_ABB_U_EXTRAP = 0, 1
 LBM_COLLISION_BGK, LBM_COLLISION_MRT = 0, 1
+LBM_ROUND_NATIVE, LBM_ROUND_DENSE = 0, 1
 
 ENTRY_POINTS = (
     "lbm_plan_create", "lbm_plan_destroy", "lbm_plan_set_kernels", "lbm_plan_get_kernels", "lbm_workspace_size", "lbm_init_geometry", "lbm_bind_geometry",
     "lbm_compact_size", "lbm_compact_bind", "lbm_set_abb_velocity", "lbm_get_abb_velocity",
-    "lbm_set_collision", "lbm_get_collision", "lbm_set_periodic_y", "lbm_set_velocity_inlet",
+    "lbm_set_rounding", "lbm_set_collision", "lbm_get_collision", "lbm_set_periodic_y", "lbm_set_velocity_inlet",
     "lbm_set_velocity_ramp", "lbm_adjoint_window",
     "lbm_forward", "lbm_step", "lbm_loss_grad", "lbm_loss_grad_noalloc", "lbm_probe_loss_grad", "lbm_spline_basis",
     "lbm_spline_profile", "lbm_spline_grad", "lbm_adjoint", "lbm_macroscopic", "lbm_darcy", "lbm_adam_step",
@@ -101,6 +102,7 @@ def load():
                 "lbm_set_abb_velocity": [vp, i32],
                 "lbm_set_collision": [vp, i32, f64, f64, f64],
                 "lbm_set_periodic_y": [vp, i32],
+                "lbm_set_rounding": [vp, i32],
                 "lbm_set_velocity_inlet": [vp, i32, f64, f64, f64],
                 "lbm_set_velocity_ramp": [vp, i32],
                 "lbm_adjoint_window": [vp, vp, vp, f64, vp, i32, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp],
@@ -284,6 +286,11 @@ def lbm_set_collision(plan: Plan, mode: int, s_e: float = 1.0, s_eps: float = 1.
            "lbm_set_collision")
 
 
+def lbm_set_rounding(plan: Plan, mode: int) -> None:
+    """How the fluid-only layout's D2Q9 FP32 kernels round: LBM_ROUND_NATIVE or LBM_ROUND_DENSE."""
+    _check(load().lbm_set_rounding(plan.handle, int(mode)), "lbm_set_rounding")
+
+
 def lbm_set_periodic_y(plan: Plan, on: bool) -> None:
     _check(load().lbm_set_periodic_y(plan.handle, 1 if on else 0), "lbm_set_periodic_y")
 
@@ -435,9 +442,20 @@ class Solver:
     r_min, r_max, target_porosity, ...), or a uint8 mask tensor (kind MASK).
 
     ``layout``: "dense" (every node stored), "compact" (fluid nodes only,
-    ``lbm_compact_bind``), or "auto" (compact for D3Q19, dense for D2Q9).
-    The default comes from the LBM_LAYOUT environment variable, else "auto".
+    ``lbm_compact_bind``), or "auto": compact, which is the faster one at
+    every size (a time step of a gradient evaluation on a GB300, dense and
+    compact: D2Q9 FP64 64x32 45.1 and 23.8 us; FP32 301x149 11.0 and 6.8,
+    512x256 10.5 and 7.7, 1024x512 27.3 and 15.5, 4096x2048 392 and 245),
+    except on a D2Q9 lattice whose environment or set_kernels() choice asks
+    for kernels that only the dense layout has.  The automatic choice rounds
+    as the dense kernels of the lattice do (LBM_ROUND_DENSE).  The
+    default comes from the LBM_LAYOUT environment variable, else "auto".
     Every array the caller sees is dense either way."""
+
+    _DENSE_ENV = ("LBM_KERNEL", "LBM_VEC", "LBM_TMA", "LBM_TMA_MIN_TILES", "LBM_TMA_VARIANT", "LBM_TMA_ROWS",
+                  "LBM_TMA_WAVES", "LBM_STEP_VARIANT", "LBM_PERSIST")
+    _DENSE_CHOICE = {"step_family", "adjoint_family", "vec", "tma_rows", "persist", "adjoint_tma_rows",
+                     "steps_per_launch", "recompute_family"}
 
     def __init__(self, q, nx, ny, nz=1, precision=4, n_steps=1, ckpt_stride=0, loss_kind=LBM_LOSS_VEC,
                  loss_norm=LBM_NORM_SUM, inlet_kind=LBM_INLET_CONST, geometry=None, device="cuda", link=None,
@@ -451,7 +469,6 @@ class Solver:
         # the library replays its T-step sweeps as CUDA graphs on a non-default stream
         self.stream = torch.cuda.Stream(device=self.device)
         p = self.plan
-        self.ws = torch.zeros(lbm_workspace_size(p), dtype=torch.uint8, device=self.device)
         if link is not None:
             self.link, self.mask = link, mask
             lbm_bind_geometry(p, link)
@@ -468,16 +485,32 @@ class Solver:
                                   fill_isolated=False)
             else:
                 lbm_init_geometry(p, self.mask, self.link, self.info, self.porosity, **(geometry or {}))
-        self.layout, self.tables = "dense", None
+        self.layout, self.tables, self.ws = "dense", None, None
         layout = layout or os.environ.get("LBM_LAYOUT", "auto")
         if layout not in ("dense", "compact", "auto"):
             raise ValueError(f"layout must be dense, compact or auto, not {layout!r}")
-        self.set_layout(("compact" if q == 19 else "dense") if layout == "auto" else layout)
+        auto = layout == "auto"
+        if auto:
+            layout = "dense" if q == 9 and any(e in os.environ for e in self._DENSE_ENV) else "compact"
+        try:
+            self.set_layout(layout)
+        except torch.cuda.OutOfMemoryError:
+            if not (auto and q == 9):
+                raise
+            self.tables = None  # an open lattice's tables can take more than its solid nodes would
+            self.set_layout("dense")
+        self._auto_2d = auto and q == 9  # until a layout is named
+        if self._auto_2d and precision == 4 and nx % 2 == 0:  # odd rows: the dense kernels round as the compact ones
+            lbm_set_rounding(p, LBM_ROUND_DENSE)
+        if self.ws is None:
+            self.ws = torch.zeros(lbm_workspace_size(p), dtype=torch.uint8, device=self.device)
 
     def set_layout(self, layout: str) -> None:
         """Switches the plan between the dense and the fluid-only state layout
         (results are the same; the workspace is reallocated)."""
         p = self.plan
+        self._auto_2d = False
+        lbm_set_rounding(p, LBM_ROUND_NATIVE)
         if layout == self.layout:
             return
         if layout == "compact":
@@ -514,7 +547,10 @@ class Solver:
         return torch.empty((self.plan.q, *self.plan.shape), dtype=self.plan.dtype, device=self.device)
 
     def set_kernels(self, **choice) -> None:
-        """lbm_plan_set_kernels, then a larger workspace where the choice needs one."""
+        """lbm_plan_set_kernels, then a larger workspace where the choice needs one.  On a D2Q9 lattice in
+        the automatic layout, naming a kernel family of the dense layout switches to that layout."""
+        if self._auto_2d and self._DENSE_CHOICE.intersection(choice):
+            self.set_layout("dense")
         lbm_plan_set_kernels(self.plan, **choice)
         self._fit_ws()
 

@@ -106,3 +106,28 @@ def test_batch_takes_both_node_block_classes():
         assert torch.equal(s.forward(r, t, 1.0), b.view_state(f, i))
         gi, gt = s.adjoint(r, t, 1.0, b.view_state(lam, i).contiguous())
         assert torch.equal(gi, b.view_inlet(g_in, i)) and torch.equal(gt, g_tau[i:i + 1])
+
+
+# rows of 4 k and of 4 k + 2 nodes: the dense layout's TMA and register kernels
+@pytest.mark.parametrize("nx,ny", [(64, 40), (66, 40), (512, 128)])
+def test_the_automatic_layout_rounds_as_the_dense_one(nx, ny):
+    m = (np.random.Generator(np.random.PCG64(nx)).uniform(size=(ny, nx)) < 0.2).astype(np.uint8)
+    T, rin, ut = 30, dev(1.0 + W.inlet_profile(ny, seed=5)), dev(W.perturbation((2, ny, nx), seed=6, scale=1e-4))
+    out = []
+    for layout in (None, "dense"):
+        s = lbm.Solver(9, nx, ny, precision=4, n_steps=T, inlet_kind=lbm.LBM_INLET_PROFILE,
+                       geometry=torch.as_tensor(m), layout=layout)
+        if layout:
+            lbm.lbm_plan_set_kernels(s.plan, step_family=lbm.LBM_FAMILY_VEC, adjoint_family=lbm.LBM_FAMILY_VEC)
+        else:
+            assert s.layout == "compact"
+        f = s.forward(rin, dev([0.8]), 1.0)
+        _, lam = s.loss_grad(f, ut)
+        out.append((f, lam, *s.adjoint(rin, dev([0.8]), 1.0, lam)))
+    (f, lam, g_in, g_tau), (fd, lamd, gd, td) = out
+    assert torch.equal(f, fd) and torch.equal(lam, lamd)
+    assert rel(g_in.cpu().numpy(), gd.cpu().numpy()) < 1e-6  # FP32 adjoint states, other compilations
+    assert rel(g_tau.cpu().numpy(), td.cpu().numpy()) < 1e-5  # FP32 warp sums over other groups of nodes
+    s = lbm.Solver(9, nx, ny, precision=4, n_steps=T, geometry=torch.as_tensor(m))
+    s.set_kernels(step_family=lbm.LBM_FAMILY_VEC)
+    assert s.layout == "dense"
