@@ -284,12 +284,15 @@ struct LdGatherT {
 
 // -------------------------------------------------------------- epilogues
 
-// y[m][off + n] = act(acc + bias[n]) in bf16.
+// y[m][off + n] = act(acc + bias[n]) in bf16; with a mask (an activation of
+// y's layout, contiguous rows of ld), the entries whose mask is not positive
+// are zero (the gradient through the ReLU that made the mask).
 struct EpAct {
     bf16* y;
     int ld, off;
     const float* bias;
     int relu;
+    const bf16* mask = nullptr;
     __device__ void set_phase(int) {}
     __device__ void store(long long m, int n, float v0, float v1) const
     {
@@ -301,7 +304,13 @@ struct EpAct {
             v0 = fmaxf(v0, 0.0f);
             v1 = fmaxf(v1, 0.0f);
         }
-        *reinterpret_cast<__nv_bfloat162*>(y + (size_t)m * ld + off + n) = __floats2bfloat162_rn(v0, v1);
+        __nv_bfloat162 o = __floats2bfloat162_rn(v0, v1);
+        if (mask) {
+            const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(mask + (size_t)m * ld + n);
+            if (!(__bfloat162float(a.x) > 0.0f)) o.x = __float2bfloat16(0.0f);
+            if (!(__bfloat162float(a.y) > 0.0f)) o.y = __float2bfloat16(0.0f);
+        }
+        *reinterpret_cast<__nv_bfloat162*>(y + (size_t)m * ld + off + n) = o;
     }
     // eight consecutive columns n .. n + 7 (n a multiple of 8): one 16-byte store
     __device__ void store8(long long m, int n, const float (&v)[8]) const
@@ -322,6 +331,17 @@ struct EpAct {
                 b = fmaxf(b, 0.0f);
             }
             o.h[j] = __floats2bfloat162_rn(a, b);
+        }
+        if (mask) {
+            union {
+                uint4 u;
+                bf16 h[8];
+            } a;
+            a.u = *reinterpret_cast<const uint4*>(mask + (size_t)m * ld + n);
+            bf16* h = reinterpret_cast<bf16*>(&o);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (!(__bfloat162float(a.h[j]) > 0.0f)) h[j] = __float2bfloat16(0.0f);
         }
         *reinterpret_cast<uint4*>(y + (size_t)m * ld + off + n) = o.u;
     }
@@ -387,6 +407,7 @@ template <class LA, class LB, class EP>
 __global__ void __launch_bounds__(kGemmThreads) k_gemm(LA la, LB lb, EP ep, long long M, int N, int K, int k_split,
                                                        int splits)
 {
+    pdl_enter();
     // operand tiles: [row][k] (k contiguous), or [k][row] for k-major loaders
     constexpr int A_BYTES = (LA::KMAJOR ? BK * (BM + 8) : BM * LDS) * 2;
     constexpr int B_BYTES = (LB::KMAJOR ? BK * (BN + 8) : BN * LDS) * 2;
@@ -516,13 +537,25 @@ struct UmmaShape {
 __device__ unsigned g_umma_status;
 constexpr unsigned kUmmaTimeout = 1u;
 constexpr uint64_t kUmmaWaitNs = 500000000ull;  // 0.5 s per wait (a copy or an MMA step takes microseconds)
-constexpr int kUmmaStages = 4;
+constexpr int kUmmaStages = 4;  // weight gradients
+
+// Stages of the convolution kernel's ring.  A tile has 9 to 36 steps, a fill
+// latency before them and an epilogue after, none of which overlap inside a
+// CTA, so what keeps an SM busy is several CTAs on it: few stages each (40 to
+// 64 KB) and three to five CTAs per SM instead of four stages and two CTAs.
+template <int KC, int BN>
+constexpr int conv_stages()
+{
+    constexpr int stage = (128 + BN) * KC * 2;
+    return stage <= 12 * 1024 ? 4 : (stage <= 16 * 1024 ? 3 : 2);
+}
 
 template <int KC, int BN>
 struct UmmaSmem {
     static constexpr int A_BYTES = 128 * KC * 2, B_BYTES = BN * KC * 2, STAGE = A_BYTES + B_BYTES;
-    static constexpr int BARS = 2 * kUmmaStages + 1;
-    static constexpr int BYTES = 1024 + kUmmaStages * STAGE + BARS * 8 + 16;  // + alignment slack
+    static constexpr int STAGES = conv_stages<KC, BN>();
+    static constexpr int BARS = 2 * STAGES + 1;
+    static constexpr int BYTES = 1024 + STAGES * STAGE + BARS * 8 + 16;  // + alignment slack
     static_assert(A_BYTES % 1024 == 0 && B_BYTES % 1024 == 0, "stage tiles keep the swizzle atoms 1024-B aligned");
 };
 
@@ -531,21 +564,25 @@ __global__ void __launch_bounds__(128, 1) k_umma_conv(const __grid_constant__ CU
                                                       const __grid_constant__ CUtensorMap tb, EP ep, UmmaShape sh)
 {
     using SM = UmmaSmem<KC, BN>;
+    constexpr int kStages = SM::STAGES;
     namespace U = umma;
     // a wait of an earlier launch gave up (flag not yet read by unet_get_status): do nothing, so that one
     // failure costs one wait limit, not one per CTA
-    if (*reinterpret_cast<volatile unsigned*>(&g_umma_status)) return;
+    if (*reinterpret_cast<volatile unsigned*>(&g_umma_status)) {
+        pdl_enter();
+        return;
+    }
     extern __shared__ unsigned char dyn[];
     const uint32_t s0 = U::smem_addr(dyn);
     unsigned char* base = dyn + ((1024u - (s0 & 1023u)) & 1023u);  // 1024-B aligned: the 128-byte swizzle atoms
-    uint64_t* full = reinterpret_cast<uint64_t*>(base + kUmmaStages * SM::STAGE);
-    uint64_t* empty = full + kUmmaStages;
-    uint64_t* done = empty + kUmmaStages;
+    uint64_t* full = reinterpret_cast<uint64_t*>(base + kStages * SM::STAGE);
+    uint64_t* empty = full + kStages;
+    uint64_t* done = empty + kStages;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int st = 0; st < kUmmaStages; ++st) {
+        for (int st = 0; st < kStages; ++st) {
             U::bar_init(&full[st], 1);
             U::bar_init(&empty[st], 1);
         }
@@ -558,6 +595,7 @@ __global__ void __launch_bounds__(128, 1) k_umma_conv(const __grid_constant__ CU
     __syncthreads();
     U::fence_after_sync();
     const uint32_t tmem = *tslot;
+    pdl_enter();  // the setup above overlaps the end of the preceding launch
     // the tile: pixels (b, y0 .. y0 + 7, x0 .. x0 + 15), columns n0 .. n0 + BN - 1 of phase ph
     const int tw = sh.W / 16, tpi = tw * (sh.H / 8);
     const int b = blockIdx.x / tpi, r = blockIdx.x % tpi;
@@ -568,9 +606,9 @@ __global__ void __launch_bounds__(128, 1) k_umma_conv(const __grid_constant__ CU
     if (warp == 0 && lane == 0) {  // producer: TMA copies into the stage ring
         int it = 0;
         for (; it < nk; ++it) {
-            const int st = it % kUmmaStages;
-            if (it >= kUmmaStages &&
-                !U::bar_wait(&empty[st], (uint32_t)(it / kUmmaStages - 1) & 1u, abort, &g_umma_status,
+            const int st = it % kStages;
+            if (it >= kStages &&
+                !U::bar_wait(&empty[st], (uint32_t)(it / kStages - 1) & 1u, abort, &g_umma_status,
                              kUmmaTimeout, kUmmaWaitNs))
                 break;
             const int tap = it / sh.kc_per_tap, kc = it - tap * sh.kc_per_tap;
@@ -581,16 +619,16 @@ __global__ void __launch_bounds__(128, 1) k_umma_conv(const __grid_constant__ CU
             U::tma_2d(sa + SM::A_BYTES, &tb, &full[st], tap * sh.C + kc * KC, ph * sh.rows_per_phase + n0);
         }
         // no copy may still be writing into shared memory when the CTA exits
-        for (int j = it > kUmmaStages ? it - kUmmaStages : 0; j < it; ++j) {
+        for (int j = it > kStages ? it - kStages : 0; j < it; ++j) {
             const uint64_t t0 = U::now_ns();
-            while (!U::bar_test(&full[j % kUmmaStages], (uint32_t)(j / kUmmaStages) & 1u))
+            while (!U::bar_test(&full[j % kStages], (uint32_t)(j / kStages) & 1u))
                 if (U::now_ns() - t0 > kUmmaWaitNs) break;
         }
     } else if (warp == 1 && lane == 0) {  // MMA issuer
         constexpr uint32_t idesc = U::idesc_bf16_m128(BN);
         for (int it = 0; it < nk; ++it) {
-            const int st = it % kUmmaStages;
-            if (!U::bar_wait(&full[st], (uint32_t)(it / kUmmaStages) & 1u, abort, &g_umma_status, kUmmaTimeout,
+            const int st = it % kStages;
+            if (!U::bar_wait(&full[st], (uint32_t)(it / kStages) & 1u, abort, &g_umma_status, kUmmaTimeout,
                              kUmmaWaitNs))
                 break;
             U::fence_after_sync();
@@ -687,7 +725,10 @@ __global__ void __launch_bounds__(128, 1) k_umma_wgrad(const __grid_constant__ C
     using WS = WgradSmem<AW, BN, BW>;
     constexpr int A_BYTES = WS::A_BYTES, STAGE = WS::STAGE;
     namespace U = umma;
-    if (*reinterpret_cast<volatile unsigned*>(&g_umma_status)) return;
+    if (*reinterpret_cast<volatile unsigned*>(&g_umma_status)) {
+        pdl_enter();
+        return;
+    }
     extern __shared__ unsigned char dyn[];
     const uint32_t s0 = U::smem_addr(dyn);
     unsigned char* base = dyn + ((1024u - (s0 & 1023u)) & 1023u);
@@ -711,6 +752,7 @@ __global__ void __launch_bounds__(128, 1) k_umma_wgrad(const __grid_constant__ C
     __syncthreads();
     U::fence_after_sync();
     const uint32_t tmem = *tslot;
+    pdl_enter();  // the setup above overlaps the end of the preceding launch
     const long long m0 = (long long)blockIdx.x * 128;
     const int n0 = blockIdx.y * BN;
     const int split = sh.up ? (int)(blockIdx.z % sh.splits) : (int)blockIdx.z;
@@ -826,40 +868,64 @@ __global__ void __launch_bounds__(128, 1) k_umma_wgrad(const __grid_constant__ C
 }
 
 // ------------------------------------------------------ elementwise kernels
+//
+// A training step at 256 x 128, batch 16, base 32 is some 110 launches of 3 to
+// 50 us: every kernel is launched with programmatic stream serialization and
+// waits for its predecessor itself, so a launch's setup overlaps the one
+// before, and what a pass would only mask, copy or convert is done where the
+// values are written (2463 -> 1930 us per step, prediction of one field 337
+// -> 210 us).
 
-__global__ void k_sum_partials(const float* __restrict__ part, long long count, int splits, long long stride,
-                               float* __restrict__ out)
+// out[i] = sum over splits of part[split * stride + i], in order.  Few outputs
+// of many splits take one warp each, lane l adding splits l, l + 32, ... in
+// order, then a fixed butterfly.
+struct Sum {
+    const float* part;
+    long long count, stride;
+    int splits;
+    float* out;
+    __host__ __device__ bool by_warp() const { return count <= 16384 && splits >= 16; }
+    __host__ unsigned blocks() const
+    {
+        return (unsigned)(by_warp() ? (count + 7) / 8
+                                    : std::max<long long>(1, std::min<long long>((count + 255) / 256, 152 * 16)));
+    }
+};
+
+__device__ __forceinline__ void add_partials(const Sum& S, unsigned block, unsigned blocks)
 {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
+    if (S.by_warp()) {
+        const long long i = (long long)block * 8 + (threadIdx.x >> 5);
+        const int lane = threadIdx.x & 31;
+        if (i >= S.count) return;
         float s = 0.0f;
-        for (int k = 0; k < splits; ++k) s += part[k * stride + i];
-        out[i] = s;
+        for (int k = lane; k < S.splits; k += 32) s += S.part[k * S.stride + i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) S.out[i] = s;
+        return;
+    }
+    for (long long i = (long long)block * 256 + threadIdx.x; i < S.count; i += (long long)blocks * 256) {
+        float s = 0.0f;
+        for (int k = 0; k < S.splits; ++k) s += S.part[k * S.stride + i];
+        S.out[i] = s;
     }
 }
 
-// The same for few outputs over many splits: one warp per output, lane l
-// adding splits l, l + 32, ... in order, then a fixed butterfly.
-__global__ void __launch_bounds__(256) k_sum_partials_warp(const float* __restrict__ part, long long count,
-                                                           int splits, long long stride, float* __restrict__ out)
+// A layer's weight gradient (blocks [0, a_blocks)) and bias gradient.
+__global__ void __launch_bounds__(256) k_sum_partials(const Sum a, const Sum b, unsigned a_blocks)
 {
-    const long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (i >= count) return;
-    float s = 0.0f;
-    for (int k = lane; k < splits; k += 32) s += part[k * stride + i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out[i] = s;
+    pdl_enter();
+    if (blockIdx.x < a_blocks) add_partials(a, blockIdx.x, a_blocks);
+    else add_partials(b, blockIdx.x - a_blocks, gridDim.x - a_blocks);
 }
 
 unsigned ew_grid(long long n);
 
-void sum_partials(cudaStream_t st, const float* part, long long count, int splits, long long stride, float* out)
+void sum_partials(cudaStream_t st, const Sum& a, const Sum& b)
 {
-    if (count <= 16384 && splits >= 16)
-        k_sum_partials_warp<<<(unsigned)((count + 7) / 8), 256, 0, st>>>(part, count, splits, stride, out);
-    else
-        k_sum_partials<<<ew_grid(count), 256, 0, st>>>(part, count, splits, stride, out);
+    const unsigned na = a.blocks(), nb = b.count ? b.blocks() : 0;
+    launch_k(true, k_sum_partials, dim3(na + nb), dim3(256), 0, st, a, b, na);
 }
 
 // Eight bf16 (16 bytes) at a time: C, row strides and channel offsets are
@@ -886,6 +952,7 @@ __device__ __forceinline__ void st8(bf16* p, const V8& v) { *reinterpret_cast<ui
 __global__ void __launch_bounds__(256) k_colsum(const bf16* __restrict__ g, long long P, int C, int ld, int off,
                                                 long long rows, float* __restrict__ part)
 {
+    pdl_enter();
     __shared__ float red[256 * 8];
     const int nv = C / 8, RG = 256 / nv, rg = threadIdx.x / nv, cv = threadIdx.x % nv;
     const long long r0 = (long long)blockIdx.x * rows, r1 = min(P, r0 + rows);
@@ -905,27 +972,13 @@ __global__ void __launch_bounds__(256) k_colsum(const bf16* __restrict__ g, long
     }
 }
 
-// out[p][c] = dy[p][off + c] * (y[p][c] > 0)
-__global__ void k_relu_grad(const bf16* __restrict__ dy, int ld_dy, int off_dy, const bf16* __restrict__ y,
-                            bf16* __restrict__ out, long long P, int C)
-{
-    const int nv = C / 8;
-    const long long n = P * nv;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / nv;
-        const int c = (int)(i - p * nv) * 8;
-        const V8 d = ld8(dy + p * ld_dy + off_dy + c), a = ld8(y + p * C + c);
-        V8 o;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) o.h[j] = __bfloat162float(a.h[j]) > 0.0f ? d.h[j] : __float2bfloat16(0.0f);
-        st8(out + p * C + c, o);
-    }
-}
-
-// 2x2 max-pool of x[B][H][W][C] (first maximum in tap order), tap index kept.
+// 2x2 max-pool of x[B][H][W][C] (first maximum in tap order), tap index kept;
+// x is copied into the second half of cat's rows of 2 C on the way (the skip
+// connection).
 __global__ void k_maxpool(const bf16* __restrict__ x, int B, int H, int W, int C, bf16* __restrict__ y,
-                          uint8_t* __restrict__ arg)
+                          uint8_t* __restrict__ arg, bf16* __restrict__ cat)
 {
+    pdl_enter();
     const int Ho = H / 2, Wo = W / 2, nv = C / 8;
     const long long n = (long long)B * Ho * Wo * nv;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -937,7 +990,9 @@ __global__ void k_maxpool(const bf16* __restrict__ x, int B, int H, int W, int C
         uint8_t bt[8];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            const V8 v = ld8(x + (((b * H) + 2 * yo + t / 2) * W + 2 * xo + t % 2) * C + c);
+            const long long p = ((b * H) + 2 * yo + t / 2) * W + 2 * xo + t % 2;
+            const V8 v = ld8(x + p * C + c);
+            st8(cat + p * 2 * C + C + c, v);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const float f = __bfloat162float(v.h[j]);
@@ -960,10 +1015,13 @@ __global__ void k_maxpool(const bf16* __restrict__ x, int B, int H, int W, int C
     }
 }
 
-// dx[B][H][W][C] = scatter of dy at the max-pool taps + skip[...][off + c] (row stride ld_s)
+// dx[B][H][W][C] = (scatter of dy at the max-pool taps + skip[...][off + c] (row stride ld_s)) * (x > 0), x the
+// pooled activation
 __global__ void k_maxpool_grad(const bf16* __restrict__ dy, const uint8_t* __restrict__ arg, int B, int H, int W,
-                               int C, const bf16* __restrict__ skip, int ld_s, int off_s, bf16* __restrict__ dx)
+                               int C, const bf16* __restrict__ skip, int ld_s, int off_s, const bf16* __restrict__ x,
+                               bf16* __restrict__ dx)
 {
+    pdl_enter();
     const int Ho = H / 2, Wo = W / 2, nv = C / 8;
     const long long n = (long long)B * H * W * nv;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -973,36 +1031,24 @@ __global__ void k_maxpool_grad(const bf16* __restrict__ dy, const uint8_t* __res
         const long long b = p / ((long long)W * H);
         const long long o = (((b * Ho) + yy / 2) * Wo + xx / 2) * C + c;
         const int t = (yy % 2) * 2 + (xx % 2);
-        const V8 d = ld8(dy + o), sk = ld8(skip + p * ld_s + off_s + c);
+        const V8 d = ld8(dy + o), sk = ld8(skip + p * ld_s + off_s + c), a = ld8(x + p * C + c);
         const uint2 ar = *reinterpret_cast<const uint2*>(arg + o);
         const uint8_t* a8 = reinterpret_cast<const uint8_t*>(&ar);
         V8 r;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const float v = (a8[j] == t ? __bfloat162float(d.h[j]) : 0.0f) + __bfloat162float(sk.h[j]);
-            r.h[j] = __float2bfloat16(v);
+            r.h[j] = __float2bfloat16(__bfloat162float(a.h[j]) > 0.0f ? v : 0.0f);
         }
         st8(dx + p * C + c, r);
     }
 }
 
-// dst[p][off + c] = src[p][c]
-__global__ void k_copy_channels(const bf16* __restrict__ src, long long P, int C, bf16* __restrict__ dst, int ld,
-                                int off)
-{
-    const int nv = C / 8;
-    const long long n = P * nv;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / nv;
-        const int c = (int)(i - p * nv) * 8;
-        st8(dst + p * ld + off + c, ld8(src + p * C + c));
-    }
-}
-
 // out[b][h] = mean_w (sum_c x[b][h][w][c] w[c] + bias): one block per row (b, h).
 __global__ void k_head(const bf16* __restrict__ x, int W, int C, const float* __restrict__ w,
-                       const float* __restrict__ bias, float* __restrict__ out)
+                       const float* __restrict__ bias, float* __restrict__ out, float* __restrict__ out2)
 {
+    pdl_enter();
     const long long row = blockIdx.x;
     float s = 0.0f;
     for (int i = threadIdx.x; i < W * C; i += blockDim.x) s += __bfloat162float(x[row * W * C + i]) * w[i % C];
@@ -1014,7 +1060,7 @@ __global__ void k_head(const bf16* __restrict__ x, int W, int C, const float* __
     if (threadIdx.x == 0) {
         float t = 0.0f;
         for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-        out[row] = t / (float)W + bias[0];
+        out[row] = out2[row] = t / (float)W + bias[0];
     }
 }
 
@@ -1022,6 +1068,7 @@ __global__ void k_head(const bf16* __restrict__ x, int W, int C, const float* __
 __global__ void k_mse(const float* __restrict__ out, const float* __restrict__ target, int n, float* __restrict__ loss,
                       float* __restrict__ gout)
 {
+    pdl_enter();
     float s = 0.0f;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const float d = out[i] - target[i];
@@ -1040,21 +1087,23 @@ __global__ void k_mse(const float* __restrict__ out, const float* __restrict__ t
     }
 }
 
-// Head backward, one block per row (b, h): dx[b][h][w][c] = gout[b][h] / W * w[c];
+// Head backward, one block per row (b, h): dx[b][h][w][c] = gout[b][h] / W * w[c] where x > 0 (x is a ReLU's output);
 // part_w[row][c] = sum_w x[b][h][w][c] gout / W.
 __global__ void __launch_bounds__(256) k_head_grad(const bf16* __restrict__ x, int W, int C,
                                                    const float* __restrict__ w, const float* __restrict__ gout,
                                                    bf16* __restrict__ dx, float* __restrict__ part_w)
 {
+    pdl_enter();
     __shared__ float red[256];
     const long long row = blockIdx.x;
     const float gr = gout[row] / (float)W;
     const int nv = C / 8;
     for (int i = threadIdx.x; i < W * nv; i += blockDim.x) {
         const int c = (i % nv) * 8;
+        const V8 a = ld8(x + row * W * C + (long long)i * 8);
         V8 o;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) o.h[j] = __float2bfloat16(gr * w[c + j]);
+        for (int j = 0; j < 8; ++j) o.h[j] = __float2bfloat16(__bfloat162float(a.h[j]) > 0.0f ? gr * w[c + j] : 0.0f);
         st8(dx + row * W * C + (long long)i * 8, o);
     }
     // part_w[row][c] = gr * sum_w x[row][w][c]: thread (group xg, channel c) adds w = xg, xg + XG, ...; the groups
@@ -1075,6 +1124,7 @@ __global__ void __launch_bounds__(256) k_head_grad(const bf16* __restrict__ x, i
 // *out = sum of v[0 .. n) (one block of 256 threads, fixed order).
 __global__ void __launch_bounds__(256) k_sum_vector(const float* __restrict__ v, int n, float* __restrict__ out)
 {
+    pdl_enter();
     __shared__ float red[256];
     float s = 0.0f;
     for (int i = threadIdx.x; i < n; i += 256) s += v[i];
@@ -1091,6 +1141,7 @@ __global__ void __launch_bounds__(256) k_sum_vector(const float* __restrict__ v,
 __global__ void k_pack(const double* __restrict__ u, const uint8_t* __restrict__ mask, int B, int H, int W,
                        float scale, bf16* __restrict__ x)
 {
+    pdl_enter();
     const long long n = (long long)B * H * W;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const long long b = i / ((long long)H * W), hw = i - b * H * W;
@@ -1103,27 +1154,66 @@ __global__ void k_pack(const double* __restrict__ u, const uint8_t* __restrict__
     }
 }
 
-// FP32 master [taps][Cin][Cout] -> fwd[co][tap * Cin + ci] and
+// Every layer's FP32 master [taps][Cin][Cout] -> fwd[co][tap * Cin + ci] and
 // bwd[ci][tap' * Cout + co] (tap' = taps - 1 - tap for a 3x3 kernel: the
 // input gradient is the correlation with the flipped kernel; for the
-// transposed convolution tap' = tap, fwd is [phase][co][ci]).
-__global__ void k_prep_weights(const float* __restrict__ w, int taps, int Cin, int Cout, int flip, int phase_major,
-                               bf16* __restrict__ fwd, bf16* __restrict__ bwd)
+// transposed convolution tap' = tap, fwd is [phase][co][ci]), and the FP32
+// copy of all parameters that biases and head are read from.  A block
+// transposes 32 x 32 (ci, co) tiles through shared memory, so that reads and
+// both writes are whole rows; layers are blockIdx.y, the copy the last one.
+// (One launch per layer with 2-byte scattered stores took 55 us at base 32.)
+constexpr int kLayers = 17;
+struct PrepLayer {
+    const float* w;
+    bf16 *fwd, *bwd;
+    int taps, cin, cout, up;
+};
+struct PrepAll {
+    PrepLayer l[kLayers];
+    const float* params;
+    float* copy;
+    long long n_params;
+};
+
+__global__ void __launch_bounds__(256) k_prep_weights(const __grid_constant__ PrepAll A)
 {
-    const long long n = (long long)taps * Cin * Cout;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int co = (int)(i % Cout), ci = (int)((i / Cout) % Cin), tap = (int)(i / ((long long)Cout * Cin));
-        const bf16 v = __float2bfloat16(w[i]);
-        if (phase_major) fwd[((long long)tap * Cout + co) * Cin + ci] = v;
-        else fwd[(long long)co * taps * Cin + (long long)tap * Cin + ci] = v;
-        const int tb = flip ? taps - 1 - tap : tap;
-        bwd[(long long)ci * taps * Cout + (long long)tb * Cout + co] = v;
+    pdl_enter();
+    if (blockIdx.y == kLayers) {
+        for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < A.n_params; i += (long long)gridDim.x * 256)
+            A.copy[i] = A.params[i];
+        return;
+    }
+    __shared__ bf16 tile[32][33];
+    const PrepLayer& L = A.l[blockIdx.y];
+    const int ti = (L.cin + 31) / 32, to = (L.cout + 31) / 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int t = blockIdx.x; t < L.taps * ti * to; t += gridDim.x) {
+        const int tap = t / (ti * to), ci0 = (t / to) % ti * 32, co0 = t % to * 32;
+        const int tb = L.up ? tap : L.taps - 1 - tap;
+        __syncthreads();
+#pragma unroll
+        for (int r = warp; r < 32; r += 8) {
+            const int ci = ci0 + r, co = co0 + lane;
+            if (ci < L.cin && co < L.cout) {
+                const bf16 v = __float2bfloat16(L.w[((long long)tap * L.cin + ci) * L.cout + co]);
+                tile[r][lane] = v;
+                L.bwd[(long long)ci * L.taps * L.cout + (long long)tb * L.cout + co] = v;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = warp; r < 32; r += 8) {
+            const int co = co0 + r, ci = ci0 + lane;
+            if (ci < L.cin && co < L.cout)
+                L.fwd[L.up ? ((long long)tap * L.cout + co) * L.cin + ci
+                           : (long long)co * L.taps * L.cin + (long long)tap * L.cin + ci] = tile[lane][r];
+        }
     }
 }
 
 __global__ void k_adam_f32(long long n, float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
                            const float* __restrict__ g, float lr, float b1, float b2, float eps, float c1, float c2)
 {
+    pdl_enter();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.0f - b1) * gi;
@@ -1191,9 +1281,10 @@ struct Layout {
     size_t bias;                                 // FP32 copy of all parameters (biases and head read from it)
     size_t ea[4], eb[4], pool[3], arg[3], cat[3], da[3], db[3];
     size_t out, gout, loss_tmp;
-    size_t gA, gB, gC, gcat[3];
+    size_t gA, gB, gcat[3];
     size_t part;                                 // split-K / column-sum partials (FP32)
     long long part_floats;
+    size_t part_b;                               // column-sum partials (FP32): up to 256 blocks x channels
     size_t total;
     int64_t n_params;
 };
@@ -1253,7 +1344,6 @@ bool make_layout(const unet_desc* d, Layout* L)
     for (int i = 0; i < 4; ++i) gmax = std::max(gmax, l.P[i] * 2 * l.c[i]);
     l.gA = act(gmax, 1);
     l.gB = act(gmax, 1);
-    l.gC = act(gmax, 1);
     l.out = o;
     o += al256(sizeof(float) * (size_t)l.B * l.H);
     l.gout = o;
@@ -1272,6 +1362,8 @@ bool make_layout(const unet_desc* d, Layout* L)
     l.part = o;
     l.part_floats = max_part;
     o += al256(sizeof(float) * (size_t)max_part);
+    l.part_b = o;
+    o += al256(sizeof(float) * 256 * (size_t)(2 * l.c[3]));
     l.total = o;
     return true;
 }
@@ -1297,7 +1389,7 @@ void gemm(cudaStream_t s, const LA& la, const LB& lb, const EP& ep, long long M,
 {
     const int k_split = ((K + splits - 1) / splits + BK - 1) / BK * BK;
     const dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)(splits * phases));
-    k_gemm<LA, LB, EP><<<grid, kGemmThreads, 0, s>>>(la, lb, ep, M, N, K, k_split, splits);
+    launch_k(true, k_gemm<LA, LB, EP>, grid, dim3(kGemmThreads), 0, s, la, lb, ep, M, N, K, k_split, splits);
 }
 
 int g_engine = UNET_ENGINE_TCGEN05;
@@ -1310,7 +1402,7 @@ bool launch_umma(cudaStream_t s, const CUtensorMap& ta, const CUtensorMap& tb, c
     static const bool attr = cudaFuncSetAttribute(k_umma_conv<KC, BN, EP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   SM::BYTES) == cudaSuccess;
     if (!attr) return false;
-    k_umma_conv<KC, BN, EP><<<grid, 128, SM::BYTES, s>>>(ta, tb, ep, sh);
+    launch_k(true, k_umma_conv<KC, BN, EP>, grid, dim3(128), SM::BYTES, s, ta, tb, ep, sh);
     return cudaGetLastError() == cudaSuccess;
 }
 
@@ -1379,7 +1471,7 @@ bool launch_wgrad(cudaStream_t s, const CUtensorMap& tx, const CUtensorMap& tg, 
     static const bool attr = cudaFuncSetAttribute(k_umma_wgrad<AW, BN, BW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   bytes) == cudaSuccess;
     if (!attr) return false;
-    k_umma_wgrad<AW, BN, BW><<<grid, 128, bytes, s>>>(tx, tg, ep, sh);
+    launch_k(true, k_umma_wgrad<AW, BN, BW>, grid, dim3(128), bytes, s, tx, tg, ep, sh);
     return cudaGetLastError() == cudaSuccess;
 }
 
@@ -1486,9 +1578,10 @@ int splits_for(long long M, long long N, long long K)
 
 // Weight and bias gradients of a 3x3 convolution with input x (ld/off) and
 // pre-activation gradient g (contiguous [P][Cout]); dx into dxo (contiguous
-// [P][Cin]) unless null.
+// [P][Cin]) unless null, masked by the positive entries of mask ([P][Cin])
+// if given.
 void conv_bwd(const Ctx& C, int layer, int wtensor, const bf16* x, int H, int W, int Cin, int ld, int off,
-              const bf16* g, int Cout, float* grad, bf16* dxo)
+              const bf16* g, int Cout, float* grad, bf16* dxo, const bf16* mask = nullptr)
 {
     const long long P = (long long)C.L.B * H * W;
     float* part = at<float>(C.ws, C.L.part);
@@ -1502,14 +1595,15 @@ void conv_bwd(const Ctx& C, int layer, int wtensor, const bf16* x, int H, int W,
         EpPartial ep{part, Cout, Mw * Cout, 0, 0, 0};
         gemm(C.s, la, lb, ep, Mw, Cout, (int)P, sp, 1);
     }
-    sum_partials(C.s, part, Mw * Cout, sp, Mw * Cout, grad + C.t[wtensor].off);
     // db[co] = sum_p g[p][co]
     const long long rows = (P + 255) / 256;
     const int nb = (int)((P + rows - 1) / rows);
-    k_colsum<<<nb, 256, 0, C.s>>>(g, P, Cout, Cout, 0, rows, part);
-    sum_partials(C.s, part, Cout, nb, Cout, grad + C.t[wtensor + 1].off);
+    float* part_b = at<float>(C.ws, C.L.part_b);
+    launch_k(true, k_colsum, dim3(nb), dim3(256), 0, C.s, g, P, Cout, Cout, 0, rows, part_b);
+    sum_partials(C.s, Sum{part, Mw * Cout, Mw * Cout, sp, grad + C.t[wtensor].off},
+                 Sum{part_b, Cout, Cout, nb, grad + C.t[wtensor + 1].off});
     if (dxo) {
-        EpAct ep2{dxo, Cin, 0, nullptr, 0};
+        EpAct ep2{dxo, Cin, 0, nullptr, 0, mask};
         if (umma_conv(C.s, g, C.L.B, H, W, Cout, Cout, 0, 9, C.wb(layer), Cin, 1, Cin, ep2)) return;
         LdIm2col<BM> la2{g, H, W, Cout, Cout, 0, 9};
         LdRows<BN> lb2{C.wb(layer), 9 * Cout, 0};
@@ -1530,9 +1624,10 @@ void up_fwd(const Ctx& C, int layer, int wtensor, const bf16* x, int Hs, int Ws,
 }
 
 // Gradients of the transposed convolution: input x (Hs x Ws, Cin), output
-// gradient in the first Cout channels of gy (row stride ld, level l).
+// gradient in the first Cout channels of gy (row stride ld, level l); dxo is
+// masked by the positive entries of mask ([P][Cin]).
 void up_bwd(const Ctx& C, int layer, int wtensor, const bf16* x, int Hs, int Ws, int Cin, const bf16* gy, int Cout,
-            int ld, float* grad, bf16* dxo)
+            int ld, float* grad, bf16* dxo, const bf16* mask)
 {
     const long long P = (long long)C.L.B * Hs * Ws;
     float* part = at<float>(C.ws, C.L.part);
@@ -1545,18 +1640,18 @@ void up_bwd(const Ctx& C, int layer, int wtensor, const bf16* x, int Hs, int Ws,
         EpPartial ep{part, Cout, 4LL * Cin * Cout, (long long)Cin * Cout, 0, 0};
         gemm(C.s, la, lb, ep, Cin, Cout, (int)P, sp, 4);
     }
-    sum_partials(C.s, part, 4LL * Cin * Cout, sp, 4LL * Cin * Cout,
-                                                               grad + C.t[wtensor].off);
     // db[co] = sum over output pixels of gy[..][co]
     const long long Po = 4 * P;
     const long long rows = (Po + 255) / 256;
     const int nb = (int)((Po + rows - 1) / rows);
-    k_colsum<<<nb, 256, 0, C.s>>>(gy, Po, Cout, ld, 0, rows, part);
-    sum_partials(C.s, part, Cout, nb, Cout, grad + C.t[wtensor + 1].off);
+    float* part_b = at<float>(C.ws, C.L.part_b);
+    launch_k(true, k_colsum, dim3(nb), dim3(256), 0, C.s, gy, Po, Cout, ld, 0, rows, part_b);
+    sum_partials(C.s, Sum{part, 4LL * Cin * Cout, 4LL * Cin * Cout, sp, grad + C.t[wtensor].off},
+                 Sum{part_b, Cout, Cout, nb, grad + C.t[wtensor + 1].off});
     // dx[p][ci] = sum_(phase, co) gy[up(p, phase)][co] W[phase][ci][co]
     LdUpGather<BM> la2{gy, Hs, Ws, Cout, ld, 0};
     LdRows<BN> lb2{C.wb(layer), 4 * Cout, 0};
-    EpAct ep2{dxo, Cin, 0, nullptr, 0};
+    EpAct ep2{dxo, Cin, 0, nullptr, 0, mask};
     gemm(C.s, la2, lb2, ep2, P, Cin, 4 * Cout, 1, 1);
 }
 
@@ -1611,8 +1706,8 @@ lbm_status unet_pack_input(const unet_desc* d, const double* d_u, const uint8_t*
     Layout L;
     if (!make_layout(d, &L) || !d_u || !d_mask || !d_x) return LBM_ERR_INVALID_ARG;
     const long long n = (long long)L.B * L.H * L.W;
-    k_pack<<<ew_grid(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(d_u, d_mask, L.B, L.H, L.W, (float)scale,
-                                                                      reinterpret_cast<bf16*>(d_x));
+    launch_k(true, k_pack, dim3(ew_grid(n)), dim3(256), 0, static_cast<cudaStream_t>(stream), d_u, d_mask, L.B, L.H, L.W,
+             (float)scale, reinterpret_cast<bf16*>(d_x));
     return cuda_status(cudaGetLastError());
 }
 
@@ -1623,15 +1718,17 @@ lbm_status unet_prepare_weights(const unet_desc* d, const float* d_params, void*
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     std::vector<int> taps, cin, cout;
     const auto t = param_tensors(d->base, &taps, &cin, &cout);
+    PrepAll A;
+    long long tiles = 0;
     for (size_t i = 0, layer = 0; i + 2 < t.size(); i += 2, ++layer) {
-        const bool up = taps[i] == 4;
-        k_prep_weights<<<ew_grid(t[i].count), 256, 0, s>>>(d_params + t[i].off, taps[i], cin[i], cout[i], up ? 0 : 1,
-                                                           up ? 1 : 0, at<bf16>(d_ws, L.wf[layer]),
-                                                           at<bf16>(d_ws, L.wb[layer]));
+        A.l[layer] = PrepLayer{d_params + t[i].off, at<bf16>(d_ws, L.wf[layer]), at<bf16>(d_ws, L.wb[layer]),
+                               taps[i], cin[i], cout[i], taps[i] == 4 ? 1 : 0};
+        tiles = std::max(tiles, (long long)taps[i] * ((cin[i] + 31) / 32) * ((cout[i] + 31) / 32));
     }
-    if (cudaMemcpyAsync(at<float>(d_ws, L.bias), d_params, sizeof(float) * (size_t)L.n_params,
-                        cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return LBM_ERR_CUDA;
+    A.params = d_params;
+    A.copy = at<float>(d_ws, L.bias);
+    A.n_params = L.n_params;
+    launch_k(true, k_prep_weights, dim3((unsigned)std::min(tiles, 304LL), kLayers + 1), dim3(256), 0, s, A);
     return cuda_status(cudaGetLastError());
 }
 
@@ -1653,10 +1750,8 @@ lbm_status unet_forward(const unet_desc* d, const uint16_t* d_x, float* d_out, v
         tensor += 2;
         if (l < 3) {
             bf16* pool = at<bf16>(d_ws, L.pool[l]);
-            k_maxpool<<<ew_grid(L.P[l + 1] * L.c[l] / 8), 256, 0, C.s>>>(eb, L.B, L.Hl[l], L.Wl[l], L.c[l], pool,
-                                                                       at<uint8_t>(d_ws, L.arg[l]));
-            k_copy_channels<<<ew_grid(L.P[l] * L.c[l] / 8), 256, 0, C.s>>>(eb, L.P[l], L.c[l], at<bf16>(d_ws, L.cat[l]),
-                                                                        2 * L.c[l], L.c[l]);
+            launch_k(true, k_maxpool, dim3(ew_grid(L.P[l + 1] * L.c[l] / 8)), dim3(256), 0, C.s, eb, L.B, L.Hl[l],
+                     L.Wl[l], L.c[l], pool, at<uint8_t>(d_ws, L.arg[l]), at<bf16>(d_ws, L.cat[l]));
             in = pool;
             cin = L.c[l];
         }
@@ -1675,9 +1770,8 @@ lbm_status unet_forward(const unet_desc* d, const uint16_t* d_x, float* d_out, v
         below = db;
     }
     float* out = at<float>(d_ws, L.out);
-    k_head<<<L.B * L.H, 256, 0, C.s>>>(below, L.W, L.c[0], C.pw(tensor), C.pw(tensor + 1), out);
-    if (cudaMemcpyAsync(d_out, out, sizeof(float) * (size_t)L.B * L.H, cudaMemcpyDeviceToDevice, C.s) != cudaSuccess)
-        return LBM_ERR_CUDA;
+    launch_k(true, k_head, dim3(L.B * L.H), dim3(256), 0, C.s, below, L.W, L.c[0], C.pw(tensor), C.pw(tensor + 1), out,
+             d_out);
     return cuda_status(cudaGetLastError());
 }
 
@@ -1691,47 +1785,48 @@ lbm_status unet_backward(const unet_desc* d, const uint16_t* d_x, const float* d
     float* gout = at<float>(d_ws, L.gout);
     float* part = at<float>(d_ws, L.part);
     const int rows = L.B * L.H;
-    k_mse<<<1, 256, 0, C.s>>>(at<float>(d_ws, L.out), d_target, rows, d_loss, gout);
+    launch_k(true, k_mse, dim3(1), dim3(256), 0, C.s, at<float>(d_ws, L.out), d_target, rows, d_loss, gout);
     // head: tensors nt-2 (w), nt-1 (b)
-    bf16* gA = at<bf16>(d_ws, L.gA);
-    bf16* gB = at<bf16>(d_ws, L.gB);
-    bf16* gC = at<bf16>(d_ws, L.gC);
+    bf16* g = at<bf16>(d_ws, L.gA);     // gradient of the pre-activation at hand
+    bf16* next = at<bf16>(d_ws, L.gB);  // ... and of the one before it
     const bf16* db0 = at<bf16>(d_ws, L.db[0]);
-    k_head_grad<<<rows, 256, 0, C.s>>>(db0, L.W, L.c[0], C.pw(nt - 2), gout, gA, part);
-    sum_partials(C.s, part, L.c[0], rows, L.c[0], d_grad + C.t[nt - 2].off);
-    k_sum_vector<<<1, 256, 0, C.s>>>(gout, rows, d_grad + C.t[nt - 1].off);
+    launch_k(true, k_head_grad, dim3(rows), dim3(256), 0, C.s, db0, L.W, L.c[0], C.pw(nt - 2), gout, g, part);
+    sum_partials(C.s, Sum{part, L.c[0], L.c[0], rows, d_grad + C.t[nt - 2].off}, Sum{});
+    launch_k(true, k_sum_vector, dim3(1), dim3(256), 0, C.s, gout, rows, d_grad + C.t[nt - 1].off);
+    // Every input gradient is masked by the ReLU it passes next in the epilogue that writes it.
     // decoder, l = 0, 1, 2 (tensors and layers counted from the end)
-    int tensor = nt - 2, layer = 16;  // 17 convolution layers, numbered in forward order
+    int tensor = nt - 2, layer = kLayers - 1;  // convolution layers, numbered in forward order
     for (int l = 0; l <= 2; ++l) {
         const int Hl = L.Hl[l], Wl = L.Wl[l], c = L.c[l];
-        // gA = dL/d(db_l)
+        const bf16* da = at<bf16>(d_ws, L.da[l]);
         tensor -= 2;  // dec{l}b
-        k_relu_grad<<<ew_grid(L.P[l] * c / 8), 256, 0, C.s>>>(gA, c, 0, at<bf16>(d_ws, L.db[l]), gB, L.P[l], c);
-        conv_bwd(C, layer--, tensor, at<bf16>(d_ws, L.da[l]), Hl, Wl, c, c, 0, gB, c, d_grad, gA);
+        conv_bwd(C, layer--, tensor, da, Hl, Wl, c, c, 0, g, c, d_grad, next, da);
+        std::swap(g, next);
         tensor -= 2;  // dec{l}a
-        k_relu_grad<<<ew_grid(L.P[l] * c / 8), 256, 0, C.s>>>(gA, c, 0, at<bf16>(d_ws, L.da[l]), gB, L.P[l], c);
         bf16* gcat = at<bf16>(d_ws, L.gcat[l]);
-        conv_bwd(C, layer--, tensor, at<bf16>(d_ws, L.cat[l]), Hl, Wl, 2 * c, 2 * c, 0, gB, c, d_grad, gcat);
+        conv_bwd(C, layer--, tensor, at<bf16>(d_ws, L.cat[l]), Hl, Wl, 2 * c, 2 * c, 0, g, c, d_grad, gcat);
         tensor -= 2;  // up{l}
         const bf16* below = l == 2 ? at<bf16>(d_ws, L.eb[3]) : at<bf16>(d_ws, L.db[l + 1]);
-        up_bwd(C, layer--, tensor, below, L.Hl[l + 1], L.Wl[l + 1], L.c[l + 1], gcat, c, 2 * c, d_grad, gA);
+        up_bwd(C, layer--, tensor, below, L.Hl[l + 1], L.Wl[l + 1], L.c[l + 1], gcat, c, 2 * c, d_grad, next, below);
+        std::swap(g, next);
     }
-    // encoder, l = 3 .. 0; gA = dL/d(eb_3) on entry
+    // encoder, l = 3 .. 0
     for (int l = 3; l >= 0; --l) {
         const int Hl = L.Hl[l], Wl = L.Wl[l], c = L.c[l];
-        if (l < 3) {  // gA = dL/d(pool_l) -> dL/d(eb_l), plus the skip gradient
-            k_maxpool_grad<<<ew_grid(L.P[l] * c / 8), 256, 0, C.s>>>(gA, at<uint8_t>(d_ws, L.arg[l]), L.B, Hl, Wl, c,
-                                                                   at<bf16>(d_ws, L.gcat[l]), 2 * c, c, gC);
-            std::swap(gA, gC);
+        if (l < 3) {  // g = dL/d(pool_l) -> dL/d(eb_l), plus the skip gradient
+            launch_k(true, k_maxpool_grad, dim3(ew_grid(L.P[l] * c / 8)), dim3(256), 0, C.s, g, at<uint8_t>(d_ws, L.arg[l]),
+                     L.B, Hl, Wl, c, at<bf16>(d_ws, L.gcat[l]), 2 * c, c, at<bf16>(d_ws, L.eb[l]), next);
+            std::swap(g, next);
         }
+        const bf16* ea = at<bf16>(d_ws, L.ea[l]);
         tensor -= 2;  // enc{l}b
-        k_relu_grad<<<ew_grid(L.P[l] * c / 8), 256, 0, C.s>>>(gA, c, 0, at<bf16>(d_ws, L.eb[l]), gB, L.P[l], c);
-        conv_bwd(C, layer--, tensor, at<bf16>(d_ws, L.ea[l]), Hl, Wl, c, c, 0, gB, c, d_grad, gA);
+        conv_bwd(C, layer--, tensor, ea, Hl, Wl, c, c, 0, g, c, d_grad, next, ea);
+        std::swap(g, next);
         tensor -= 2;  // enc{l}a
-        k_relu_grad<<<ew_grid(L.P[l] * c / 8), 256, 0, C.s>>>(gA, c, 0, at<bf16>(d_ws, L.ea[l]), gB, L.P[l], c);
         const int cin = l == 0 ? UNET_IN_CHANNELS : L.c[l - 1];
         const bf16* in = l == 0 ? reinterpret_cast<const bf16*>(d_x) : at<bf16>(d_ws, L.pool[l - 1]);
-        conv_bwd(C, layer--, tensor, in, Hl, Wl, cin, cin, 0, gB, c, d_grad, l == 0 ? nullptr : gA);
+        conv_bwd(C, layer--, tensor, in, Hl, Wl, cin, cin, 0, g, c, d_grad, l == 0 ? nullptr : next);
+        std::swap(g, next);
     }
     return cuda_status(cudaGetLastError());
 }
@@ -1741,8 +1836,8 @@ lbm_status unet_adam(int64_t n, float* d_params, float* d_m, float* d_v, const f
 {
     if (n < 1 || t < 1 || !d_params || !d_m || !d_v || !d_grad) return LBM_ERR_INVALID_ARG;
     const float c1 = 1.0f - powf(beta1, (float)t), c2 = 1.0f - powf(beta2, (float)t);
-    k_adam_f32<<<ew_grid(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(n, d_params, d_m, d_v, d_grad, lr, beta1,
-                                                                          beta2, eps, c1, c2);
+    launch_k(true, k_adam_f32, dim3(ew_grid(n)), dim3(256), 0, static_cast<cudaStream_t>(stream), n, d_params, d_m, d_v,
+             d_grad, lr, beta1, beta2, eps, c1, c2);
     return cuda_status(cudaGetLastError());
 }
 
