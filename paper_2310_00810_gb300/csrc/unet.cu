@@ -506,6 +506,164 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm(LA la, LB lb, EP ep, long
         }
 }
 
+// ------------------------------------------------------- the input layer
+//
+// The first convolution gathers 8 channels: 16 bytes per pixel and tap, too
+// short a row for the tensor-memory kernels' boxes, and K = 72.  Both of its
+// products move little more than its output (33 MB at 256 x 128, batch 16,
+// base 32), so these kernels feed mma.sync straight from memory, without the
+// general gather's index arithmetic: forward 72 -> 12 us, weight gradient
+// 93 -> 17 us.
+
+// y = relu(conv3x3(x) + bias): a warp takes 16 pixels of a row x 32 output
+// channels; an A fragment's registers are 4-byte loads (two channels of a
+// pixel, two taps per 16-deep step), the weights stay in registers.  The
+// steps run over K in order, as k_gemm's do.  Width a multiple of 16, output
+// channels of 32.
+__global__ void __launch_bounds__(128) k_conv_in(const bf16* __restrict__ x, const bf16* __restrict__ wf,
+                                                 const float* __restrict__ bias, int B, int H, int W, int Cout,
+                                                 bf16* __restrict__ y)
+{
+    pdl_enter();
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, n0 = blockIdx.y * 32;
+    uint32_t b[5][4][2];
+    float bs[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const bf16* w = wf + (size_t)(n0 + 8 * j + g) * 72 + 2 * t;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            b[k][j][0] = *reinterpret_cast<const uint32_t*>(w + 16 * k);
+            b[k][j][1] = k < 4 ? *reinterpret_cast<const uint32_t*>(w + 16 * k + 8) : 0u;
+        }
+        bs[j][0] = bias[n0 + 8 * j + 2 * t];
+        bs[j][1] = bias[n0 + 8 * j + 2 * t + 1];
+    }
+    const int per_row = W / 16;
+    const long long groups = (long long)B * H * per_row;
+    for (long long q = (long long)blockIdx.x * 4 + (threadIdx.x >> 5); q < groups; q += (long long)gridDim.x * 4) {
+        const int x0 = (int)(q % per_row) * 16, row = (int)(q / per_row), yy0 = row % H;
+        uint32_t a[5][4];
+#pragma unroll
+        for (int tap = 0; tap < 10; ++tap) {
+            const int dy = tap / 3 - 1, dx = tap % 3 - 1;
+            const bool in = tap < 9 && yy0 + dy >= 0 && yy0 + dy < H;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {  // pixels g and g + 8
+                const int xx = x0 + g + 8 * h + dx;
+                uint32_t v = 0u;
+                if (in && xx >= 0 && xx < W)
+                    v = *reinterpret_cast<const uint32_t*>(x + ((size_t)(row + dy) * W + xx) * 8 + 2 * t);
+                a[tap / 2][(tap & 1) * 2 + h] = v;
+            }
+        }
+        float acc[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[j][c] = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) mma16816(acc[j], a[k], b[k][j]);
+        }
+        // a quad holds 4 x 8 channels of a pixel in pairs: transposed, lane t holds channels 8 t .. 8 t + 7
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t u[4], o[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const __nv_bfloat162 p = __floats2bfloat162_rn(fmaxf(acc[j][2 * h] + bs[j][0], 0.0f),
+                                                               fmaxf(acc[j][2 * h + 1] + bs[j][1], 0.0f));
+                u[j] = *reinterpret_cast<const uint32_t*>(&p);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int s = t ^ r;
+                const uint32_t v = __shfl_xor_sync(0xffffffffu, s == 0 ? u[0] : s == 1 ? u[1] : s == 2 ? u[2] : u[3], r);
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (c == s) o[c] = v;
+            }
+            *reinterpret_cast<uint4*>(y + ((size_t)row * W + x0 + g + 8 * h) * Cout + n0 + 8 * t) =
+                make_uint4(o[0], o[1], o[2], o[3]);
+        }
+    }
+}
+
+// part[block][72][Cout] of its weight gradient: a block takes strips of one
+// image row (at most 256 pixels), the three input rows around it and 32
+// channels of g in shared memory; K is the pixels, a tap pair an A tile's 16
+// rows (transposed fragments of 8 pixels x 8 channels), and the eight warps'
+// sums are added in order.
+constexpr int kInStrip = 256;
+__global__ void __launch_bounds__(256) k_wgrad_in(const bf16* __restrict__ x, const bf16* __restrict__ g, int B, int H,
+                                                  int W, int Cout, float* __restrict__ part)
+{
+    __shared__ __align__(16) bf16 xs[3][kInStrip + 2][8];
+    __shared__ __align__(16) bf16 gs[kInStrip][40];
+    __shared__ float red[72 * 32];
+    pdl_enter();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 3, rr = lane & 7, n0 = blockIdx.y * 32;
+    const int strips = (W + kInStrip - 1) / kInStrip;
+    float acc[5][4][4];
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[i][j][c] = 0.0f;
+    for (long long s = blockIdx.x; s < (long long)B * H * strips; s += gridDim.x) {
+        const int row = (int)(s / strips), x0 = (int)(s % strips) * kInStrip, n = min(kInStrip, W - x0), y = row % H;
+        __syncthreads();
+        for (int i = threadIdx.x; i < 3 * (n + 2); i += 256) {
+            const int dy = i / (n + 2) - 1, c = i % (n + 2), xx = x0 + c - 1;
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (y + dy >= 0 && y + dy < H && xx >= 0 && xx < W)
+                v = *reinterpret_cast<const uint4*>(x + ((size_t)(row + dy) * W + xx) * 8);
+            *reinterpret_cast<uint4*>(&xs[dy + 1][c][0]) = v;
+        }
+        for (int i = threadIdx.x; i < 4 * n; i += 256)
+            *reinterpret_cast<uint4*>(&gs[i / 4][8 * (i % 4)]) =
+                *reinterpret_cast<const uint4*>(g + ((size_t)row * W + x0 + i / 4) * Cout + n0 + 8 * (i % 4));
+        __syncthreads();
+        for (int k0 = warp * 16; k0 < n; k0 += 128) {  // n is a multiple of 16
+            uint32_t b[4][2];
+#pragma unroll
+            for (int j = 0; j < 4; j += 2) {
+                uint32_t r4[4];
+                ldmatrix_x4_trans(r4, &gs[k0 + (q & 1) * 8 + rr][8 * j + (q & 2) * 4]);
+                b[j][0] = r4[0];
+                b[j][1] = r4[1];
+                b[j + 1][0] = r4[2];
+                b[j + 1][1] = r4[3];
+            }
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const int tap = min(2 * i + (q & 1), 8);  // the tenth "tap" repeats the ninth; its rows are left out
+                uint32_t a[4];
+                ldmatrix_x4_trans(a, &xs[tap / 3][k0 + (q & 2) * 4 + rr + tap % 3][0]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) mma16816(acc[i][j], a, b[j]);
+            }
+        }
+    }
+    for (int w = 0; w < 8; ++w) {
+        __syncthreads();
+        if (warp != w) continue;
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int m = 16 * i + (lane >> 2) + 8 * (c >> 1), nn = 8 * j + 2 * (lane & 3) + (c & 1);
+                    if (m < 72) red[m * 32 + nn] = w ? red[m * 32 + nn] + acc[i][j][c] : acc[i][j][c];
+                }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 72 * 32; i += 256)
+        part[((size_t)blockIdx.x * 72 + i / 32) * Cout + n0 + i % 32] = red[i];
+}
+
 // ------------------------------------------------ tcgen05 convolution GEMM
 //
 // The convolution GEMMs whose A operand is an image gathered through taps
@@ -541,29 +699,31 @@ constexpr int kUmmaStages = 4;  // weight gradients
 
 // Stages of the convolution kernel's ring.  A tile has 9 to 36 steps, a fill
 // latency before them and an epilogue after, none of which overlap inside a
-// CTA, so what keeps an SM busy is several CTAs on it: few stages each (40 to
-// 64 KB) and three to five CTAs per SM instead of four stages and two CTAs.
+// CTA, so what keeps an SM busy on a large grid is several CTAs on it: few
+// stages each (40 to 64 KB, DEPTH 0) and three to five CTAs per SM.  A grid of
+// at most one CTA per SM has only its ring to hide each copy's latency:
+// eight stages (DEPTH 2); up to two per SM, four (DEPTH 1).
 template <int KC, int BN>
-constexpr int conv_stages()
+constexpr int conv_stages(int depth)
 {
     constexpr int stage = (128 + BN) * KC * 2;
-    return stage <= 12 * 1024 ? 4 : (stage <= 16 * 1024 ? 3 : 2);
+    return depth == 2 ? 8 : depth == 1 ? 4 : (stage <= 12 * 1024 ? 4 : (stage <= 16 * 1024 ? 3 : 2));
 }
 
-template <int KC, int BN>
+template <int KC, int BN, int DEPTH>
 struct UmmaSmem {
     static constexpr int A_BYTES = 128 * KC * 2, B_BYTES = BN * KC * 2, STAGE = A_BYTES + B_BYTES;
-    static constexpr int STAGES = conv_stages<KC, BN>();
+    static constexpr int STAGES = conv_stages<KC, BN>(DEPTH);
     static constexpr int BARS = 2 * STAGES + 1;
     static constexpr int BYTES = 1024 + STAGES * STAGE + BARS * 8 + 16;  // + alignment slack
     static_assert(A_BYTES % 1024 == 0 && B_BYTES % 1024 == 0, "stage tiles keep the swizzle atoms 1024-B aligned");
 };
 
-template <int KC, int BN, class EP>
+template <int KC, int BN, int DEPTH, class EP>
 __global__ void __launch_bounds__(128, 1) k_umma_conv(const __grid_constant__ CUtensorMap ta,
                                                       const __grid_constant__ CUtensorMap tb, EP ep, UmmaShape sh)
 {
-    using SM = UmmaSmem<KC, BN>;
+    using SM = UmmaSmem<KC, BN, DEPTH>;
     constexpr int kStages = SM::STAGES;
     namespace U = umma;
     // a wait of an earlier launch gave up (flag not yet read by unet_get_status): do nothing, so that one
@@ -957,8 +1117,19 @@ __global__ void __launch_bounds__(256) k_colsum(const bf16* __restrict__ g, long
     const int nv = C / 8, RG = 256 / nv, rg = threadIdx.x / nv, cv = threadIdx.x % nv;
     const long long r0 = (long long)blockIdx.x * rows, r1 = min(P, r0 + rows);
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (long long r = r0 + rg; r < r1; r += RG) {
-        const V8 v = ld8(g + r * ld + off + 8 * cv);
+    const bf16* p = g + off + 8 * cv;
+    long long r = r0 + rg;
+    for (; r + 3 * RG < r1; r += 4 * RG) {  // four loads in flight
+        V8 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = ld8(p + (r + u * RG) * ld);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(v[u].h[j]);
+    }
+    for (; r < r1; r += RG) {
+        const V8 v = ld8(p + r * ld);
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(v.h[j]);
     }
@@ -1051,7 +1222,14 @@ __global__ void k_head(const bf16* __restrict__ x, int W, int C, const float* __
     pdl_enter();
     const long long row = blockIdx.x;
     float s = 0.0f;
-    for (int i = threadIdx.x; i < W * C; i += blockDim.x) s += __bfloat162float(x[row * W * C + i]) * w[i % C];
+    const bf16* xr = x + row * W * C;
+    if (blockDim.x % C == 0) {  // one channel per thread: no division, and the loads run ahead of the sum
+        const float wc = w[threadIdx.x % C];
+#pragma unroll 8
+        for (int i = threadIdx.x; i < W * C; i += blockDim.x) s += __bfloat162float(xr[i]) * wc;
+    } else {
+        for (int i = threadIdx.x; i < W * C; i += blockDim.x) s += __bfloat162float(xr[i]) * w[i % C];
+    }
     __shared__ float red[32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -1158,7 +1336,7 @@ __global__ void k_pack(const double* __restrict__ u, const uint8_t* __restrict__
 // bwd[ci][tap' * Cout + co] (tap' = taps - 1 - tap for a 3x3 kernel: the
 // input gradient is the correlation with the flipped kernel; for the
 // transposed convolution tap' = tap, fwd is [phase][co][ci]), and the FP32
-// copy of all parameters that biases and head are read from.  A block
+// copy of the biases and the head.  A block
 // transposes 32 x 32 (ci, co) tiles through shared memory, so that reads and
 // both writes are whole rows; layers are blockIdx.y, the copy the last one.
 // (One launch per layer with 2-byte scattered stores took 55 us at base 32.)
@@ -1179,8 +1357,12 @@ __global__ void __launch_bounds__(256) k_prep_weights(const __grid_constant__ Pr
 {
     pdl_enter();
     if (blockIdx.y == kLayers) {
-        for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < A.n_params; i += (long long)gridDim.x * 256)
-            A.copy[i] = A.params[i];
+        const int l = blockIdx.x;  // layer l's bias; the last block: the head
+        if (l > kLayers) return;
+        const long long i0 = l < kLayers ? A.l[l].w - A.params + (long long)A.l[l].taps * A.l[l].cin * A.l[l].cout
+                                         : A.n_params - A.l[0].cout - 1;
+        const int n = l < kLayers ? A.l[l].cout : A.l[0].cout + 1;
+        for (int i = threadIdx.x; i < n; i += 256) A.copy[i0 + i] = A.params[i0 + i];
         return;
     }
     __shared__ bf16 tile[32][33];
@@ -1278,13 +1460,13 @@ struct Layout {
     int Hl[4], Wl[4];
     long long P[4];                              // pixels per level (all samples)
     size_t wf[17], wb[17];                       // bf16 operand layouts of the 17 convolution layers (forward order)
-    size_t bias;                                 // FP32 copy of all parameters (biases and head read from it)
+    size_t bias;                                 // FP32 copy of the biases and the head, at their offsets
     size_t ea[4], eb[4], pool[3], arg[3], cat[3], da[3], db[3];
     size_t out, gout, loss_tmp;
     size_t gA, gB, gcat[3];
     size_t part;                                 // split-K / column-sum partials (FP32)
     long long part_floats;
-    size_t part_b;                               // column-sum partials (FP32): up to 256 blocks x channels
+    size_t part_b;                               // column-sum partials (FP32): up to kColsumBlocks blocks x channels
     size_t total;
     int64_t n_params;
 };
@@ -1363,7 +1545,7 @@ bool make_layout(const unet_desc* d, Layout* L)
     l.part_floats = max_part;
     o += al256(sizeof(float) * (size_t)max_part);
     l.part_b = o;
-    o += al256(sizeof(float) * 256 * (size_t)(2 * l.c[3]));
+    o += al256(sizeof(float) * 608 * (size_t)(2 * l.c[3]));
     l.total = o;
     return true;
 }
@@ -1394,27 +1576,39 @@ void gemm(cudaStream_t s, const LA& la, const LB& lb, const EP& ep, long long M,
 
 int g_engine = UNET_ENGINE_TCGEN05;
 
+template <int KC, int BN, int DEPTH, class EP>
+bool launch_umma_depth(cudaStream_t s, const CUtensorMap& ta, const CUtensorMap& tb, const EP& ep, const UmmaShape& sh,
+                       dim3 grid)
+{
+    using SM = UmmaSmem<KC, BN, DEPTH>;
+    static const bool attr = cudaFuncSetAttribute(k_umma_conv<KC, BN, DEPTH, EP>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, SM::BYTES) == cudaSuccess;
+    if (!attr) return false;
+    launch_k(true, k_umma_conv<KC, BN, DEPTH, EP>, grid, dim3(128), SM::BYTES, s, ta, tb, ep, sh);
+    return cudaGetLastError() == cudaSuccess;
+}
+
 template <int KC, int BN, class EP>
 bool launch_umma(cudaStream_t s, const CUtensorMap& ta, const CUtensorMap& tb, const EP& ep, const UmmaShape& sh,
-                 dim3 grid)
+                 dim3 grid, int sms)
 {
-    using SM = UmmaSmem<KC, BN>;
-    static const bool attr = cudaFuncSetAttribute(k_umma_conv<KC, BN, EP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  SM::BYTES) == cudaSuccess;
-    if (!attr) return false;
-    launch_k(true, k_umma_conv<KC, BN, EP>, grid, dim3(128), SM::BYTES, s, ta, tb, ep, sh);
-    return cudaGetLastError() == cudaSuccess;
+    if constexpr (BN <= 64) {  // wider tiles are chosen for large grids only
+        const long long ctas = (long long)grid.x * grid.y * grid.z;
+        if (ctas <= sms) return launch_umma_depth<KC, BN, 2>(s, ta, tb, ep, sh, grid);
+        if (ctas <= 2LL * sms) return launch_umma_depth<KC, BN, 1>(s, ta, tb, ep, sh, grid);
+    }
+    return launch_umma_depth<KC, BN, 0>(s, ta, tb, ep, sh, grid);
 }
 
 template <int KC, class EP>
 bool launch_umma_bn(int bn, cudaStream_t s, const CUtensorMap& ta, const CUtensorMap& tb, const EP& ep,
-                    const UmmaShape& sh, dim3 grid)
+                    const UmmaShape& sh, dim3 grid, int sms)
 {
     switch (bn) {
-    case 32: return launch_umma<KC, 32>(s, ta, tb, ep, sh, grid);
-    case 64: return launch_umma<KC, 64>(s, ta, tb, ep, sh, grid);
-    case 128: return launch_umma<KC, 128>(s, ta, tb, ep, sh, grid);
-    default: return launch_umma<KC, 256>(s, ta, tb, ep, sh, grid);
+    case 32: return launch_umma<KC, 32>(s, ta, tb, ep, sh, grid, sms);
+    case 64: return launch_umma<KC, 64>(s, ta, tb, ep, sh, grid, sms);
+    case 128: return launch_umma<KC, 128>(s, ta, tb, ep, sh, grid, sms);
+    default: return launch_umma<KC, 256>(s, ta, tb, ep, sh, grid, sms);
     }
 }
 
@@ -1460,7 +1654,8 @@ bool umma_conv(cudaStream_t s, const bf16* x, int Bimg, int H, int W, int C, int
         return false;
     UmmaShape sh{H, W, C, taps, (C + KC - 1) / KC, N, rows_per_phase};
     const dim3 grid((unsigned)tiles_m, (unsigned)((N + bn - 1) / bn), (unsigned)phases);
-    return KC == 64 ? launch_umma_bn<64>(bn, s, ta, tb, ep, sh, grid) : launch_umma_bn<32>(bn, s, ta, tb, ep, sh, grid);
+    return KC == 64 ? launch_umma_bn<64>(bn, s, ta, tb, ep, sh, grid, sms)
+                    : launch_umma_bn<32>(bn, s, ta, tb, ep, sh, grid, sms);
 }
 
 template <int AW, int BN, int BW>
@@ -1554,11 +1749,27 @@ int umma_wgrad(cudaStream_t s, const bf16* x, int Bimg, int H, int W, int Cin, i
     return ok ? (int)sp : 0;
 }
 
+// Rows per block of a column sum: four blocks per SM, at least 64 rows each.
+constexpr int kColsumBlocks = 608;
+long long colsum_rows(long long P) { return std::max(64LL, (P + kColsumBlocks - 1) / kColsumBlocks); }
+
+// Whether the input layer's own kernels take a convolution.
+bool input_layer(const Ctx&, int W, int Cin, int Cout, int ld)
+{
+    return g_engine == UNET_ENGINE_TCGEN05 && Cin == UNET_IN_CHANNELS && ld == Cin && Cout % 32 == 0 && W % 16 == 0;
+}
+
 // conv3x3 (+bias, ReLU) of x (level geometry H x W, Cin channels at ld/off) into y (contiguous Cout).
 void conv_fwd(const Ctx& C, int layer, int wtensor, const bf16* x, int H, int W, int Cin, int ld, int off, bf16* y,
               int Cout)
 {
     const long long P = (long long)C.L.B * H * W;
+    if (input_layer(C, W, Cin, Cout, ld)) {
+        const long long groups = P / 16;
+        launch_k(true, k_conv_in, dim3((unsigned)std::min((groups + 3) / 4, 152LL * 8), Cout / 32), dim3(128), 0, C.s, x,
+                 C.wf(layer), C.pw(wtensor + 1), C.L.B, H, W, Cout, y);
+        return;
+    }
     EpAct ep{y, Cout, 0, C.pw(wtensor + 1), 1};
     if (umma_conv(C.s, x, C.L.B, H, W, Cin, ld, off, 9, C.wf(layer), Cout, 1, Cout, ep)) return;
     LdIm2col<BM> la{x, H, W, Cin, ld, off, 9};
@@ -1587,7 +1798,14 @@ void conv_bwd(const Ctx& C, int layer, int wtensor, const bf16* x, int H, int W,
     float* part = at<float>(C.ws, C.L.part);
     // dW[(tap, ci)][co] = sum_p x[p + tap][ci] g[p][co]
     const long long Mw = 9LL * Cin;
-    int sp = umma_wgrad(C.s, x, C.L.B, H, W, Cin, ld, off, g, Cout, part, C.L.part_floats);
+    int sp = 0;
+    if (input_layer(C, W, Cin, Cout, ld)) {
+        const long long strips = (long long)C.L.B * H * ((W + kInStrip - 1) / kInStrip);
+        sp = (int)std::min(std::min(strips, 304LL), C.L.part_floats / (Mw * Cout));
+        launch_k(true, k_wgrad_in, dim3(sp, Cout / 32), dim3(256), 0, C.s, x, g, C.L.B, H, W, Cout, part);
+    } else {
+        sp = umma_wgrad(C.s, x, C.L.B, H, W, Cin, ld, off, g, Cout, part, C.L.part_floats);
+    }
     if (!sp) {
         sp = splits_for(Mw, Cout, P);
         LdGatherT<BM> la{x, H, W, Cin, ld, off, 9, 0, 0};
@@ -1596,7 +1814,7 @@ void conv_bwd(const Ctx& C, int layer, int wtensor, const bf16* x, int H, int W,
         gemm(C.s, la, lb, ep, Mw, Cout, (int)P, sp, 1);
     }
     // db[co] = sum_p g[p][co]
-    const long long rows = (P + 255) / 256;
+    const long long rows = colsum_rows(P);
     const int nb = (int)((P + rows - 1) / rows);
     float* part_b = at<float>(C.ws, C.L.part_b);
     launch_k(true, k_colsum, dim3(nb), dim3(256), 0, C.s, g, P, Cout, Cout, 0, rows, part_b);
@@ -1642,7 +1860,7 @@ void up_bwd(const Ctx& C, int layer, int wtensor, const bf16* x, int Hs, int Ws,
     }
     // db[co] = sum over output pixels of gy[..][co]
     const long long Po = 4 * P;
-    const long long rows = (Po + 255) / 256;
+    const long long rows = colsum_rows(Po);
     const int nb = (int)((Po + rows - 1) / rows);
     float* part_b = at<float>(C.ws, C.L.part_b);
     launch_k(true, k_colsum, dim3(nb), dim3(256), 0, C.s, gy, Po, Cout, ld, 0, rows, part_b);
@@ -1728,7 +1946,7 @@ lbm_status unet_prepare_weights(const unet_desc* d, const float* d_params, void*
     A.params = d_params;
     A.copy = at<float>(d_ws, L.bias);
     A.n_params = L.n_params;
-    launch_k(true, k_prep_weights, dim3((unsigned)std::min(tiles, 304LL), kLayers + 1), dim3(256), 0, s, A);
+    launch_k(true, k_prep_weights, dim3((unsigned)std::max(std::min(tiles, 304LL), kLayers + 1LL), kLayers + 1), dim3(256), 0, s, A);
     return cuda_status(cudaGetLastError());
 }
 
