@@ -237,15 +237,14 @@ void set_dense(lbm_plan* p)
     } while (0)
 
 // The last launch of a sweep: stream-only from the internal state cur into
-// the caller's dense array.  Solid nodes are zeroed first: the compact layout
-// writes fluid nodes only, and the dense kernels skip 32-byte sectors that
-// hold only solid nodes.
+// the caller's dense array, solid entries zero.  The dense kernels skip 32-byte
+// sectors that hold only solid nodes, so the array is zeroed before them.
 lbm_status final_stream(const lbm_plan* p, const void* cur, void* d_f, const Bc& bc, const double* tau,
                         cudaStream_t s, int lin = kLayoutNatural)
 {
+    if (p->info.cmp.nf) return stream_dense_launch(p->info, cur, d_f, bc, s, lin);
     if (cudaMemsetAsync(d_f, 0, p->dense_state_bytes, s) != cudaSuccess) return LBM_ERR_CUDA;
-    if (!p->info.cmp.nf) return step_launch(p->info, kStreamOnly, cur, d_f, bc, tau, s);
-    return step_launch_cmp(p->info, kStreamOnly, cur, d_f, false, true, bc, tau, s, lin);
+    return step_launch(p->info, kStreamOnly, cur, d_f, bc, tau, s);
 }
 
 // One stream-collide launch of a sweep producing g^t from g^{t-1}: the

@@ -301,6 +301,12 @@ __global__ void k_batch_finish(const BInst* __restrict__ insts, const double* __
     }
 }
 
+__global__ void k_batch_unit_weights(double* __restrict__ w, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) w[i] = 1.0;
+}
+
 // The same in the fluid-only layout: instance i's dL/domega partials are the
 // warp slots [k0 / 32, (k0 + nf + 31) / 32) of the packed compact kernels,
 // summed in the order a single compact plan sums its own.
@@ -311,8 +317,7 @@ __global__ void k_batch_finish_cmp(const BCmpInst* __restrict__ insts, const dou
     const BCmpInst I = insts[blockIdx.x];
     const long long w0 = I.k0 >> 5, nw = (I.nf + 31) >> 5;
     double v = 0.0;
-    for (long long u = threadIdx.x; u < nw; u += blockDim.x) v += partial[w0 + u];
-    v = block_sum(v, threadIdx.x, blockDim.x);
+    v = block_reduce_array(partial + w0, nw);
     const int n_acc = I.g.ny * I.g.nz;
     double gs = 0.0;
     if (I.n_in == 1) {
@@ -720,9 +725,13 @@ lbm_status lbm_batch_loss_grad(lbm_batch* b, const void* d_f, const double* d_u_
 #define LBM_BATCH_LOSS(Q, T)                                                                                        \
     do {                                                                                                            \
         constexpr int V = batch_vec<Q, T>();                                                                           \
-        k_batch_loss<Q, T, V><<<grid, block, 0, s>>>(I, U, nu, static_cast<const T*>(d_f), d_u_target, d_roi, kind, \
-                                                     wgt, static_cast<T*>(d_lambda), part, 1);                      \
-        k_batch_reduce<<<b->n, kReduceThreads, 0, s>>>(I, part, 1, mean, wgt, st);                                 \
+        if (mean) { /* the ROI count */                                                                           \
+            k_batch_loss<Q, T, V><<<grid, block, 0, s>>>(I, U, nu, static_cast<const T*>(d_f), d_u_target, d_roi,   \
+                                                         kind, wgt, static_cast<T*>(d_lambda), part, 1);            \
+            k_batch_reduce<<<b->n, kReduceThreads, 0, s>>>(I, part, 1, mean, wgt, st);                             \
+        } else {                                                                                                    \
+            k_batch_unit_weights<<<(b->n + 255) / 256, 256, 0, s>>>(wgt, b->n);                                     \
+        }                                                                                                           \
         k_batch_loss<Q, T, V><<<grid, block, 0, s>>>(I, U, nu, static_cast<const T*>(d_f), d_u_target, d_roi, kind, \
                                                      wgt, static_cast<T*>(d_lambda), part, 0);                      \
         k_batch_reduce<<<b->n, kReduceThreads, 0, s>>>(I, part, 0, mean, d_loss, st);                              \

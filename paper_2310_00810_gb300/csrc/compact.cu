@@ -1257,6 +1257,38 @@ __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
     add_warp_partial<T>(dom, k < (int32_t)c.nf, k, partial);
 }
 
+// The last launch of a sweep of a single lattice: stream-only into the
+// caller's dense array, one thread per dense node, solid entries zero, so that
+// every sector is written once and whole (written by compact node, after a
+// memset, 512x256x256 took 1008 + 380 us).
+template <int Q, typename T, int IN>
+__global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
+    k_stream_dense(const T* src, T* __restrict__ dst, Cmp c, CmpBlk lat, const BCmpInst* __restrict__ insts,
+                   const int32_t* __restrict__ cmap, long long N, Bc tmpl)
+{
+    pdl_enter();
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= N) return;
+    const int32_t k = __ldg(cmap + n);
+    T v[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = T(0);
+    if (k >= 0) {
+        const Node nd = node_of(k, c, lat, nullptr);
+        if (!nd.bnd()) {
+            Neighbours<Q> nb;
+            if (IN == kInGather) window_neighbours<Q>(nb, c, lat, k, nd.pos);
+            pull_interior<Q, T, IN, IN == kInLocal>(v, src, k, (uint32_t)c.nf, nb);
+        } else {
+            int32_t code[Q];
+            const Wall wall = boundary_codes<Q>(code, nd, c, insts, tmpl);
+            pull_table<Q, T, IN, IN == kInLocal>(v, src, k, wall, (size_t)c.nf, code, tmpl, insts, false);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) dst[(size_t)i * (size_t)N + n] = v[i];
+}
+
 // The caller's dense arrays (packed, for a batch) -> the compact state
 // (ADD: added to it).  SWAP: into the swapped lambda layout (lambda_d(x) to
 // (x - c_d, opp(d)) where that node is fluid), the layout of lambda^t at odd
@@ -1649,6 +1681,27 @@ lbm_status step_launch_cmp(const PlanInfo& p, int mode, const void* src, void* d
 {
     if (p.cmp.nf == 0) return LBM_OK;
     return step_any(single_args(p, bc.status), mode, src, dst, dense_in, dense_out, bc, tau, s, lin, lout);
+}
+
+template <int Q, typename T>
+static void launch_stream_dense(const PlanInfo& p, const void* src, void* dst, const Bc& bc, cudaStream_t s, int lin)
+{
+    const dim3 grid((unsigned)((p.geo.N + kCmpThreads - 1) / kCmpThreads)), block(kCmpThreads);
+    auto go = [&](auto kernel) {
+        launch_k(p.pdl, kernel, grid, block, 0, s, static_cast<const T*>(src), static_cast<T*>(dst), p.cmp, p.cmp_lat,
+                 p.cmp_inst, p.cmp_map, p.geo.N, bc);
+    };
+    if (lin == kLayoutSwapped) go(k_stream_dense<Q, T, kInLocal>);
+    else go(k_stream_dense<Q, T, kInGather>);
+}
+
+lbm_status stream_dense_launch(const PlanInfo& p, const void* src, void* dst, const Bc& bc, cudaStream_t s, int lin)
+{
+    if (p.q == 9 && p.prec == 4) launch_stream_dense<9, float>(p, src, dst, bc, s, lin);
+    else if (p.q == 9) launch_stream_dense<9, double>(p, src, dst, bc, s, lin);
+    else if (p.prec == 4) launch_stream_dense<19, float>(p, src, dst, bc, s, lin);
+    else launch_stream_dense<19, double>(p, src, dst, bc, s, lin);
+    return cuda_status(cudaGetLastError());
 }
 
 lbm_status adjoint_launch_cmp(const PlanInfo& p, int t0, const void* gprev, const void* lam_in, void* lam_out,
