@@ -1372,8 +1372,13 @@ BCmpArgs single_args(const PlanInfo& p, uint32_t* status)
 // blocks spread the few warps evenly over the SMs (128x64 to 512x256 D2Q9:
 // 64 threads 6.3 to 7.7 us per time step of a gradient evaluation, 256
 // threads 6.7 to 8.4); above it 128 were fastest on D2Q9 (1024x512: 15.5 us,
-// 16.7 with 256) and 256 on D3Q19 (128x64x64: 24.1 us, 24.6 with 128).
-unsigned cmp_threads(int q, long long nf) { return nf < 100000 ? 64 : (q == 9 ? 128 : 256); }
+// 16.7 with 256) and 256 on D3Q19 (128x64x64: 24.1 us, 24.6 with 128).  FP64
+// small lattices take single warps: the SM with the most of them sets the time.
+unsigned cmp_threads(int q, int prec, long long nf)
+{
+    if (nf < 100000) return prec == 8 ? 32 : 64;
+    return q == 9 ? 128 : 256;
+}
 
 // The pipelined kernels, from four nodes per resident thread: D2Q9 FP32
 // 2048x1024 takes 58.9 us per time step of a gradient evaluation with them
@@ -1419,7 +1424,7 @@ void launch_step_as(const BCmpArgs& a, int mode, const void* src, void* dst, boo
 {
     const T* x = static_cast<const T*>(src);
     T* y = static_cast<T*>(dst);
-    const unsigned threads = cmp_threads(Q, a.c.nf);
+    const unsigned threads = cmp_threads(Q, (int)sizeof(T), a.c.nf);
     const CmpOrder ord = cmp_order(a, threads, tmpl.t_level);
     const dim3 grid(ord.n), block(threads);
     const bool swap_in = lin == kLayoutSwapped, swap_out = lout == kLayoutSwapped;
@@ -1473,7 +1478,7 @@ template <int Q, typename T, int IN, int OUT, bool DENSE_ROUND>
 void launch_adjoint_as(const BCmpArgs& a, int t0, const T* gp, const T* li, T* lo, const Bc& tmpl, const double* tau,
                        double* grad_acc, double* partial, cudaStream_t s)
 {
-    const unsigned threads = cmp_threads(Q, a.c.nf);
+    const unsigned threads = cmp_threads(Q, (int)sizeof(T), a.c.nf);
     const CmpOrder ord = cmp_order(a, threads, tmpl.t_level);
     auto go = [&](auto kernel) {
         launch_k(a.pdl, kernel, dim3(ord.n), dim3(threads), 0, s, gp, li, lo, a.c, a.lat, a.insts, a.blks, tmpl,
