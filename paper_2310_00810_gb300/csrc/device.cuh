@@ -60,8 +60,8 @@ __device__ __forceinline__ T cdot(int i, const T (&u)[3])
 
 // Where the equilibrium and its adjoint are evaluated by opposite pairs and
 // moments: FP64, which runs at about two lanes per SM and clock, so that its
-// kernels are as fast as they have few operations (64x32 D2Q9: 7.9 us per time
-// step of a gradient evaluation by direction and in 64-thread blocks, 6.0 so
+// kernels are as fast as they have few operations (64x32 D2Q9: 23.7 us per time
+// level of a gradient evaluation by direction and in 64-thread blocks, 18.0 so
 // and in 32-thread blocks).  FP32 keeps the sums by direction: its layouts
 // round alike term by term, and on D3Q19 pairs gave 1 to 3 %.
 template <typename T>

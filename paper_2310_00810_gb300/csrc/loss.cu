@@ -102,7 +102,10 @@ __global__ void k_loss_weight(const double* __restrict__ partial, int nb, double
 }
 
 // Per node: u from shifted f^T; loss term; lambda^T_k = sum_a dL/du_a (c_ka - u_a) / rho.
-// MEAN: the terms carry *weight, else 1.  One FP64 partial per block.
+// MEAN: the terms carry *weight, else 1.  One FP64 partial per block.  Bound by
+// FP64 on lattices in cache (128x64x64 D3Q19 FP32: 18 us, 24 without the list)
+// and by memory on large ones (512x256x256: 1584 us with a block sum per 128
+// nodes, 1400 so, for 6.0 GB).
 template <int Q, typename T, int KIND, bool MEAN>
 __global__ void __launch_bounds__(kChunkThreads)
     k_loss(const T* __restrict__ f, const double* __restrict__ ut, const uint8_t* __restrict__ roi, Geo g,
@@ -113,57 +116,58 @@ __global__ void __launch_bounds__(kChunkThreads)
     const long long N = g.N;
     const double wgt = MEAN ? *weight : 1.0;
     double term = 0.0;
-    for (long long base = (long long)blockIdx.x * chunk; base < N; base += (long long)gridDim.x * chunk) {
-        const int cnt = chunk_list(
-            list, base, base + chunk < N ? base + chunk : N, [&](long long n) { return !(g.link[n] & kLinkSolid) && (!roi || roi[n]); },
-            [&](long long n) {
+    auto node = [&](long long n) {
+        T v[Q];
 #pragma unroll
-                for (int k = 0; k < Q; ++k) lam[(long long)k * N + n] = T(0);
-            });
-        for (int i = threadIdx.x; i < cnt; i += kChunkThreads) {
-            const long long n = base + list[i];
-            T v[Q];
+        for (int j = 0; j < Q; ++j) v[j] = f[(long long)j * N + n];
+        double t[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-            for (int j = 0; j < Q; ++j) v[j] = f[(long long)j * N + n];
-            double t[3] = {0.0, 0.0, 0.0};
+        for (int a = 0; a < L::D; ++a) t[a] = ut[(long long)a * N + n];
+        T drho, rho, u[3];
+        moments<Q, T>(v, drho, rho, u);
+        double du[3] = {0.0, 0.0, 0.0};
+        if (KIND == LBM_LOSS_VEC) {
 #pragma unroll
-            for (int a = 0; a < L::D; ++a) t[a] = ut[(long long)a * N + n];
-            T drho, rho, u[3];
-            moments<Q, T>(v, drho, rho, u);
-            double du[3] = {0.0, 0.0, 0.0};
-            if (KIND == LBM_LOSS_VEC) {
-#pragma unroll
-                for (int a = 0; a < L::D; ++a) {
-                    const double e = (double)u[a] - t[a];
-                    term += MEAN ? wgt * e * e : e * e;
-                    du[a] = MEAN ? 2.0 * wgt * e : e;
-                }
-            } else {
-                double uu = 0.0, tt = 0.0;
-#pragma unroll
-                for (int a = 0; a < L::D; ++a) {
-                    uu += (double)u[a] * (double)u[a];
-                    tt += t[a] * t[a];
-                }
-                const double un = sqrt(uu);
-                const double e = un - sqrt(tt);
+            for (int a = 0; a < L::D; ++a) {
+                const double e = (double)u[a] - t[a];
                 term += MEAN ? wgt * e * e : e * e;
-                if (uu != 0.0)
-#pragma unroll
-                    for (int a = 0; a < L::D; ++a) du[a] = (MEAN ? 2.0 * wgt : 1.0) * e * (double)u[a] / un;
+                du[a] = MEAN ? 2.0 * wgt * e : e;
             }
-            T dv[3];
+        } else {
+            double uu = 0.0, tt = 0.0;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) dv[a] = MEAN ? T(du[a]) : T(2) * T(du[a]);  // doubling is exact
-            const T inv = T(1) / rho;
-#pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                T s = 0;
-#pragma unroll
-                for (int a = 0; a < L::D; ++a) s += dv[a] * (T(L::c(k, a)) - u[a]);
-                lam[(long long)k * N + n] = s * inv;
+            for (int a = 0; a < L::D; ++a) {
+                uu += (double)u[a] * (double)u[a];
+                tt += t[a] * t[a];
             }
+            const double un = sqrt(uu);
+            const double e = un - sqrt(tt);
+            term += MEAN ? wgt * e * e : e * e;
+            if (uu != 0.0)
+#pragma unroll
+                for (int a = 0; a < L::D; ++a) du[a] = (MEAN ? 2.0 * wgt : 1.0) * e * (double)u[a] / un;
         }
+        T dv[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) dv[a] = MEAN ? T(du[a]) : T(2) * T(du[a]);  // doubling is exact
+        const T inv = T(1) / rho;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            T s = 0;
+#pragma unroll
+            for (int a = 0; a < L::D; ++a) s += dv[a] * (T(L::c(k, a)) - u[a]);
+            lam[(long long)k * N + n] = s * inv;
+        }
+    };
+    auto active = [&](long long n) { return !(g.link[n] & kLinkSolid) && (!roi || roi[n]); };
+    auto idle = [&](long long n) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) lam[(long long)k * N + n] = T(0);
+    };
+    for (long long base = (long long)blockIdx.x * chunk; base < N; base += (long long)gridDim.x * chunk) {
+        const long long end = base + chunk < N ? base + chunk : N;
+        const int cnt = chunk_list(list, base, end, active, idle);
+        for (int i = threadIdx.x; i < cnt; i += kChunkThreads) node(base + list[i]);
     }
     const double bs = block_sum(term, threadIdx.x, blockDim.x);
     if (threadIdx.x == 0) partial[blockIdx.x] = bs;
@@ -443,7 +447,8 @@ lbm_status finish_gradients_launch(const PlanInfo& p, const double* grad_acc, co
 
 // ------------------------------------------------------- macroscopic
 
-// FP64 moments.  A component's quotient is its product with the reciprocal and
+// FP64 moments; bound by FP64 (128x64x64 D3Q19, half of it solid: 115 us
+// without the list, 56 with it).  A component's quotient is its product with the reciprocal and
 // one step of Markstein's correction (IBM J. Res. Dev. 34, 1990), within an ulp
 // of the division; the ends of the exponent range take the division itself.
 template <int Q, typename T>
