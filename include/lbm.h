@@ -283,10 +283,14 @@ LBM_API lbm_status lbm_compact_bind(lbm_plan* plan, int64_t n_fluid, void* d_tab
  *                     terms of dL/dtau from P = 1 + 3 c.u + ..., so that a
  *                     lattice's results do not depend on which of the two
  *                     layouts an automatic choice gives it
- * With LBM_ABB_U_EXTRAP the dense layout has neither kernel and the setting has
- * no effect.  Cached CUDA graphs are dropped on a change.  Errors: INVALID_ARG
+ *   LBM_ROUND_DENSE_NODE  as the dense layout's one-node-per-thread kernels
+ *                     (odd row lengths): 1 / tau rounded from FP64, and the
+ *                     terms of dL/dtau summed to FP64 accuracy
+ * With LBM_ABB_U_EXTRAP or the MRT collision the dense layout runs the
+ * one-node-per-thread kernels, and LBM_ROUND_DENSE gives 1 / tau and those
+ * sums as they do.  Cached CUDA graphs are dropped on a change.  Errors: INVALID_ARG
  * for an unknown mode. */
-enum { LBM_ROUND_NATIVE = 0, LBM_ROUND_DENSE = 1 };
+enum { LBM_ROUND_NATIVE = 0, LBM_ROUND_DENSE = 1, LBM_ROUND_DENSE_NODE = 2 };
 LBM_API lbm_status lbm_set_rounding(lbm_plan* plan, int32_t mode);
 
 /* T steps from rest (f = w_i, rho = 1: init_field of section 2.2), keeping

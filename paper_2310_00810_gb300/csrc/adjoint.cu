@@ -18,7 +18,7 @@
 //        G_a = sum over this node's Eq. 6 links i of lambda_i 2 w_i rho_w (9 (c_i.u) c_ia - 3 u_a)
 //      (Eq. 6 uses the node's own u at time t);
 //   4. dL/domega += sum_j mu_j (f^eq_j - f_j)  (one FP64 partial per block,
-//      accumulated in place across steps: fixed order, no atomics);
+//      accumulated in place across steps by one addition per launch: fixed order);
 //      dL/drho_w(y, z) += sum over Eq. 6 inlet links of lambda_i 2 w_i (1 + 4.5 (c_i.u)^2 - 1.5 u.u)
 //      (one owner thread per inlet node, accumulated in place across steps).
 // With the extrapolated Eq. 6 velocity a second, per-row pass adds what the
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kStepThreads)
     const uint32_t lw = live ? __ldg(g.link + n) : kLinkSolid;
     const bool fluid = !(lw & kLinkSolid), xin = x == 0, xout = x == g.nx - 1;
     const double rw = fluid && (xin || xout) ? wall_density(bc, g, xin, y, z) : 1.0;
-    const T omega = T(1) / T(*tau);
+    const T omega = relaxation_rate<T>(*tau, bc.wide);
     pdl_enter();
     T dom = T(0);
     T lamv[Q];
@@ -95,11 +95,10 @@ __global__ void __launch_bounds__(kStepThreads)
     if (stores_node(fluid, live, g, sizeof(T) == 4))
 #pragma unroll
         for (int k = 0; k < Q; ++k) lam_out[(long long)k * N + n] = lamv[k];
-    // dL/domega: warp sums in T (FP64 is slow on this part), the block's in FP64
+    // dL/domega: warp sums without FP64 lanes (warp_total), the block's in FP64
     __shared__ double s_part[kStepThreads / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dom += __shfl_xor_sync(0xffffffffu, dom, o);
-    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = (double)dom;
+    const double ws = warp_total(dom, bc.wide);
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = ws;
     __syncthreads();
     if (threadIdx.x == 0) {
         double bs = 0.0;
@@ -173,10 +172,12 @@ static void launch(const PlanInfo& p, int t0, const void* gprev, const void* lam
     const T* gp = static_cast<const T*>(gprev);
     const T* li = static_cast<const T*>(lam_in);
     T* lo = static_cast<T*>(lam_out);
+    Bc b = bc;
+    b.wide = !DENSE_ROUND;  // DENSE_ROUND stands in for the TMA kernels
     if (t0)
-        launch_k(p.pdl, k_adjoint<Q, T, true, DENSE_ROUND>, dim3(p.grid), dim3(kStepThreads), 0, s, gp, li, lo, p.geo, bc, tau, grad_acc, partial);
+        launch_k(p.pdl, k_adjoint<Q, T, true, DENSE_ROUND>, dim3(p.grid), dim3(kStepThreads), 0, s, gp, li, lo, p.geo, b, tau, grad_acc, partial);
     else
-        launch_k(p.pdl, k_adjoint<Q, T, false, DENSE_ROUND>, dim3(p.grid), dim3(kStepThreads), 0, s, gp, li, lo, p.geo, bc, tau, grad_acc, partial);
+        launch_k(p.pdl, k_adjoint<Q, T, false, DENSE_ROUND>, dim3(p.grid), dim3(kStepThreads), 0, s, gp, li, lo, p.geo, b, tau, grad_acc, partial);
 }
 
 lbm_status adjoint_launch(const PlanInfo& plan, int t_is_zero, const void* gprev, const void* lam_in, void* lam_out,

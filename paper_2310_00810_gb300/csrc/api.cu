@@ -159,6 +159,8 @@ Bc make_bc(const lbm_plan* p, const double* rho_in, double rho_out, void* ws)
     bc.test_stall = p->info.test_stall ? 1 : 0;
     bc.ramp_steps = p->info.vel_inlet ? p->info.ramp_steps : 0;
     bc.ramp = inlet_ramp(bc.ramp_steps, 0);
+    // the dense layout runs the extrapolated u_w and the MRT collision on its one-node-per-thread kernels
+    bc.wide = p->info.node_round || (p->info.dense_round && (p->info.mrt || p->info.uw_extrap)) ? 1 : 0;
     for (int a = 0; a < 3; ++a) {
         bc.u_in[a] = p->info.u_in[a];
         bc.mrt_rates[a] = p->info.mrt_rates[a];
@@ -476,8 +478,9 @@ lbm_status lbm_set_collision(lbm_plan* p, int32_t mode, double s_e, double s_eps
 
 lbm_status lbm_set_rounding(lbm_plan* p, int32_t mode)
 {
-    if (!p || (mode != LBM_ROUND_NATIVE && mode != LBM_ROUND_DENSE)) return LBM_ERR_INVALID_ARG;
+    if (!p || mode < LBM_ROUND_NATIVE || mode > LBM_ROUND_DENSE_NODE) return LBM_ERR_INVALID_ARG;
     p->info.dense_round = mode == LBM_ROUND_DENSE ? 1 : 0;
+    p->info.node_round = mode == LBM_ROUND_DENSE_NODE ? 1 : 0;
     drop_graphs(p);
     return LBM_OK;
 }

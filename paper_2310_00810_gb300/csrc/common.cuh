@@ -48,6 +48,7 @@ struct Bc {
     char uw_extrap = 0;    // 1: Eq. 6 takes u_w extrapolated to the pressure plane (LBM_ABB_U_EXTRAP)
     char mrt = 0;          // 1: D2Q9 MRT collision (Eq. 16-18) with the free rates of mrt_rates
     char vel_inlet = 0;    // 1: velocity inlet through x = -1/2 (moving-wall bounce-back) with u_in
+    char wide = 0;         // 1: FP32 kernels round 1 / tau from FP64 and sum dL/domega over a warp to FP64 accuracy
     double rho_out;
     uint32_t* status;      // device status word (bounded waits latch LBM_ERR_TIMEOUT here)
     uint32_t wait_us = 2000000u;  // time bound of each mbarrier wait of the TMA kernels, in microseconds
@@ -130,6 +131,7 @@ struct PlanInfo {
     int uw_extrap;    // 1: Eq. 6 with the extrapolated wall velocity (one-node-per-thread or fluid-only kernels)
     int mrt;          // 1: D2Q9 MRT collision (one-node-per-thread or fluid-only kernels)
     int dense_round;  // 1: LBM_ROUND_DENSE
+    int node_round;   // 1: LBM_ROUND_DENSE_NODE
     int tma_named;    // 1: the environment sets from which size the TMA kernels are used
     int vel_inlet;    // 1: velocity inlet instead of Eq. 6 at x = -1/2 (fluid-only kernels)
     double u_in[3];   // its velocity

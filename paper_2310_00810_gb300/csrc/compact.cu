@@ -647,8 +647,8 @@ __device__ __forceinline__ void apply_eq6(T (&v)[Q], const T* src, int32_t k, co
     const T drw = T(wall.rw - 1.0), rwT = T(wall.rw);
     // Opposite links together: a node has one of each pair (nx > 1), and a warp
     // holds nodes of both sides.  These warps decide how long a small lattice's
-    // step takes (64x32 FP64: 18.0 us per time level of a gradient evaluation
-    // link by link here and in the adjoint, 15.2 so).
+    // step takes (64x32 FP64: 2.8 of 18.0 us per time level of a gradient
+    // evaluation less than link by link here and in the adjoint).
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         if (L::c(i, 0) != 1) continue;
@@ -877,20 +877,19 @@ __device__ __forceinline__ T adjoint_node(const T (&f)[Q], const T (&mu)[Q], con
     return dom;
 }
 
-// One FP64 partial per warp (its sum in T), accumulated in place across time
-// steps: no block barrier, so a warp that finishes early frees its slot at
+// One FP64 partial per warp (its sum in T, or to FP64 accuracy where wide),
+// accumulated in place across time steps: no block barrier, so a warp that finishes early frees its slot at
 // once instead of waiting for the slowest warp of the block.  The warp of
 // compact node k owns slot k >> 5 (lane 0 holds the warp's first node).  The
 // addition is a reduction at the L2 cache, whose result nothing waits for:
 // each slot has one per launch, so the order of additions is the order of the
 // launches.
 template <typename T>
-__device__ __forceinline__ void add_warp_partial(T dom, bool live, long long k, double* __restrict__ partial)
+__device__ __forceinline__ void add_warp_partial(T dom, bool live, long long k, double* __restrict__ partial,
+                                                 bool wide)
 {
-    T dw = dom;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dw += __shfl_xor_sync(0xffffffffu, dw, o);
-    if ((threadIdx.x & 31) == 0 && live) atomicAdd(partial + (k >> 5), (double)dw);
+    const double dw = warp_total(dom, wide);
+    if ((threadIdx.x & 31) == 0 && live) atomicAdd(partial + (k >> 5), dw);
 }
 
 // Reverse of the extrapolated Eq. 6 velocity in the compact layout: the
@@ -992,7 +991,7 @@ __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
         return;
     }
     const BCmpInst* I = insts + nd.blk.inst;
-    const T omega = T(1) / T(tau[nd.blk.inst]);
+    const T omega = relaxation_rate<T>(tau[nd.blk.inst], Q == 9 && tmpl.wide);
     const bool side = tmpl.side_u != nullptr;
     T v[Q];
     Wall wall;
@@ -1118,7 +1117,7 @@ __device__ __forceinline__ void pipe_step_node(const PipeArgs<T>& A, unsigned b)
         window_neighbours<Q>(nb, A.c, nd.blk, nd.k, nd.pos);
         pull_interior<Q, T, kInGather, false>(v, A.src, nd.k, (uint32_t)A.c.nf, nb);
     }
-    collide_any<Q, T, DENSE_ROUND>(v, T(1) / T(A.tau[nd.blk.inst]), A.tmpl);
+    collide_any<Q, T, DENSE_ROUND>(v, relaxation_rate<T>(A.tau[nd.blk.inst], Q == 9 && A.tmpl.wide), A.tmpl);
     store_node<Q, T, kOutOwn>(A.out, v, nd, A.c, I);
 }
 
@@ -1134,7 +1133,7 @@ __global__ void __launch_bounds__(kPipeThreads, MINB) k_step_cmp_pipe(const __gr
     Ahead<Q, T, BATCH> a;
     a.start(A, b);
     int cur = a.k2.inst;
-    T omega = T(1) / T(A.tau[cur]);
+    T omega = relaxation_rate<T>(A.tau[cur], Q == 9 && A.tmpl.wide);
     pdl_enter();
     const uint32_t NF = (uint32_t)A.c.nf;
     auto fetch = [&](T(&v)[Q]) {
@@ -1145,7 +1144,7 @@ __global__ void __launch_bounds__(kPipeThreads, MINB) k_step_cmp_pipe(const __gr
     auto update = [&](const CmpBlk& blk, T(&v)[Q]) {
         if (BATCH && blk.inst != cur) {
             cur = blk.inst;
-            omega = T(1) / T(A.tau[cur]);
+            omega = relaxation_rate<T>(A.tau[cur], Q == 9 && A.tmpl.wide);
         }
         collide_any<Q, T, DENSE_ROUND>(v, omega, A.tmpl);
         const int32_t k = a.node(blk);
@@ -1193,9 +1192,9 @@ __device__ __forceinline__ void pipe_adjoint_node(const PipeArgs<T>& A, unsigned
             window_neighbours<Q>(nb, A.c, nd.blk, nd.k, nd.pos);
             pull_adjoint<Q, T, false, kInGather, false>(f, mu, A.src, A.lam_in, nd.k, (uint32_t)A.c.nf, nb);
         }
-        dom = adjoint_node<Q, T, kOutOwn, DENSE_ROUND>(f, mu, G, A.out, nd, A.c, A.tmpl, T(1) / T(A.tau[nd.blk.inst]));
+        dom = adjoint_node<Q, T, kOutOwn, DENSE_ROUND>(f, mu, G, A.out, nd, A.c, A.tmpl, relaxation_rate<T>(A.tau[nd.blk.inst], Q == 9 && A.tmpl.wide));
     }
-    add_warp_partial<T>(dom, nd.k < (int32_t)A.c.nf, nd.k, A.partial);
+    add_warp_partial<T>(dom, nd.k < (int32_t)A.c.nf, nd.k, A.partial, Q == 9 && A.tmpl.wide);
 }
 
 template <int Q, typename T, bool BATCH, bool DENSE_ROUND, int MINB>
@@ -1210,7 +1209,7 @@ __global__ void __launch_bounds__(kPipeThreads, MINB) k_adjoint_cmp_pipe(const _
     Ahead<Q, T, BATCH> a;
     a.start(A, b);
     int cur = a.k2.inst;
-    T omega = T(1) / T(A.tau[cur]);
+    T omega = relaxation_rate<T>(A.tau[cur], Q == 9 && A.tmpl.wide);
     pdl_enter();
     const uint32_t NF = (uint32_t)A.c.nf;
     auto fetch = [&](T(&f)[Q], T(&mu)[Q]) {
@@ -1221,13 +1220,13 @@ __global__ void __launch_bounds__(kPipeThreads, MINB) k_adjoint_cmp_pipe(const _
     auto update = [&](const CmpBlk& blk, T(&f)[Q], T(&mu)[Q]) {
         if (BATCH && blk.inst != cur) {
             cur = blk.inst;
-            omega = T(1) / T(A.tau[cur]);
+            omega = relaxation_rate<T>(A.tau[cur], Q == 9 && A.tmpl.wide);
         }
         const T G[3] = {T(0), T(0), T(0)};
         Node nd;
         nd.k = a.node(blk);
         const T dom = adjoint_node<Q, T, kOutOwn, DENSE_ROUND>(f, mu, G, A.out, nd, A.c, A.tmpl, omega);
-        add_warp_partial<T>(dom, true, nd.k, A.partial);
+        add_warp_partial<T>(dom, true, nd.k, A.partial, Q == 9 && A.tmpl.wide);
     };
     T f0[Q], m0[Q], f1[Q], m1[Q];
     fetch(f0, m0);
@@ -1269,7 +1268,7 @@ __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
         for (int i = 0; i < Q; ++i) f[i] = T(0);
     }
     T omega = T(0);
-    if (nd.live()) omega = T(1) / T(tau[nd.blk.inst]);
+    if (nd.live()) omega = relaxation_rate<T>(tau[nd.blk.inst], Q == 9 && tmpl.wide);
     if (nd.interior()) {
         Neighbours<Q> nb;
         if (IN == kInGather) window_neighbours<Q>(nb, c, nd.blk, k, nd.pos);
@@ -1286,7 +1285,7 @@ __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
     }
     T dom = T(0);
     if (nd.live()) dom = adjoint_node<Q, T, OUT, DENSE_ROUND>(f, mu, G, lam_out, nd, c, tmpl, omega);
-    add_warp_partial<T>(dom, k < (int32_t)c.nf, k, partial);
+    add_warp_partial<T>(dom, k < (int32_t)c.nf, k, partial, Q == 9 && tmpl.wide);
 }
 
 // The last launch of a sweep of a single lattice: stream-only into the

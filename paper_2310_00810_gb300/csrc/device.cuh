@@ -7,6 +7,49 @@
 
 namespace lbm {
 
+// omega = 1 / tau.  wide: rounded from the FP64 quotient, without an FP64
+// division in every thread (an FP32 quotient corrected by its residual,
+// accurate to 2^-47 before the last rounding).
+template <typename T>
+__device__ __forceinline__ T relaxation_rate(double tau, bool wide)
+{
+    const T t = T(tau), w = T(1) / t;
+    if constexpr (sizeof(T) == 4) {
+        if (wide) {
+            const float lo = (float)(tau - (double)t);  // tau = t + lo
+            const float r = fmaf(fmaf(-lo, w, fmaf(-t, w, 1.0f)), w, w);
+            if (isfinite(r)) return r;
+        }
+    }
+    return w;
+}
+
+// The sum of one term per lane, valid in lane 0: in T, or (wide, FP32) to the
+// accuracy of an FP64 sum as pairs of FP32 numbers: each addition keeps its
+// rounding error exactly (Knuth's two-sum).  FP64 lanes would cost 80 cycles
+// of an SM's FP64 pipe per warp.
+template <typename T>
+__device__ __forceinline__ double warp_total(T v, bool wide)
+{
+    if constexpr (sizeof(T) == 4) {
+        if (wide) {
+            float hi = v, lo = 0.0f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+                const float s = hi + h2, b = s - hi;
+                lo += l2 + ((hi - (s - b)) + (h2 - b));
+                hi = s;
+            }
+            return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return (double)v;
+}
+
+
 template <int Q>
 __host__ __device__ constexpr long long link_offset(int i, int nx, long long plane)
 {
@@ -61,8 +104,9 @@ __device__ __forceinline__ T cdot(int i, const T (&u)[3])
 // Where the equilibrium and its adjoint are evaluated by opposite pairs and
 // moments: FP64, which runs at about two lanes per SM and clock, so that its
 // kernels are as fast as they have few operations (64x32 D2Q9: 23.7 us per time
-// level of a gradient evaluation by direction and in 64-thread blocks, 18.0 so
-// and in 32-thread blocks).  FP32 keeps the sums by direction: its layouts
+// level of a gradient evaluation by direction, in 64-thread blocks and Eq. 6
+// link by link; 16.8 so, in 32-thread blocks and with opposite Eq. 6 links
+// together).  FP32 keeps the sums by direction: its layouts
 // round alike term by term, and on D3Q19 pairs gave 1 to 3 %.
 template <typename T>
 constexpr bool kByPairs = std::is_same<T, double>::value;

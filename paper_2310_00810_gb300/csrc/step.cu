@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(kStepThreads) k_step(const T* src, T* dst, Geo
     const uint32_t lw = live ? __ldg(g.link + n) : kLinkSolid;
     const bool fluid = !(lw & kLinkSolid);
     const double rw = fluid && (x == 0 || x == g.nx - 1) ? wall_density(bc, g, x == 0, y, z) : 1.0;
-    const T omega = MODE == kStreamOnly ? T(0) : T(1) / T(*tau);
+    const T omega = MODE == kStreamOnly ? T(0) : relaxation_rate<T>(*tau, bc.wide);
     pdl_enter();
     T v[Q];
 #pragma unroll
@@ -85,10 +85,12 @@ lbm_status step_launch(const PlanInfo& plan, int mode, const void* src, void* ds
     const PlanInfo p = with_family(plan, family);
     if (step_launch_tma(p, mode, src, dst, bc, tau, s)) return cuda_status(cudaGetLastError());
     if (step_launch_vec(p, mode, src, dst, bc, tau, s)) return cuda_status(cudaGetLastError());
-    if (p.q == 9 && p.prec == 4) launch<9, float>(p, mode, src, dst, bc, tau, s);
-    else if (p.q == 9 && p.prec == 8) launch<9, double>(p, mode, src, dst, bc, tau, s);
-    else if (p.q == 19 && p.prec == 4) launch<19, float>(p, mode, src, dst, bc, tau, s);
-    else if (p.q == 19 && p.prec == 8) launch<19, double>(p, mode, src, dst, bc, tau, s);
+    Bc b = bc;
+    b.wide = bc.uw_extrap || bc.mrt || !auto_scalar(plan, plan.step_family);  // else it stands in for the TMA kernels
+    if (p.q == 9 && p.prec == 4) launch<9, float>(p, mode, src, dst, b, tau, s);
+    else if (p.q == 9 && p.prec == 8) launch<9, double>(p, mode, src, dst, b, tau, s);
+    else if (p.q == 19 && p.prec == 4) launch<19, float>(p, mode, src, dst, b, tau, s);
+    else if (p.q == 19 && p.prec == 8) launch<19, double>(p, mode, src, dst, b, tau, s);
     else return LBM_ERR_UNSUPPORTED;
     return cuda_status(cudaGetLastError());
 }

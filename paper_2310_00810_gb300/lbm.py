@@ -29,7 +29,7 @@ LBM_LINK_SOLID = 0x80000000
 LBM_FAMILY_AUTO, LBM_FAMILY_SCALAR, LBM_FAMILY_VEC, LBM_FAMILY_TMA = 0, 1, 2, 3
 LBM_ABB_U_NODE, LBM_ABB_U_EXTRAP = 0, 1
 LBM_COLLISION_BGK, LBM_COLLISION_MRT = 0, 1
-LBM_ROUND_NATIVE, LBM_ROUND_DENSE = 0, 1
+LBM_ROUND_NATIVE, LBM_ROUND_DENSE, LBM_ROUND_DENSE_NODE = 0, 1, 2
 
 ENTRY_POINTS = (
     "lbm_plan_create", "lbm_plan_destroy", "lbm_plan_set_kernels", "lbm_plan_get_kernels", "lbm_workspace_size", "lbm_init_geometry", "lbm_bind_geometry",
@@ -287,7 +287,7 @@ def lbm_set_collision(plan: Plan, mode: int, s_e: float = 1.0, s_eps: float = 1.
 
 
 def lbm_set_rounding(plan: Plan, mode: int) -> None:
-    """How the fluid-only layout's D2Q9 FP32 kernels round: LBM_ROUND_NATIVE or LBM_ROUND_DENSE."""
+    """How the fluid-only layout's D2Q9 FP32 kernels round: LBM_ROUND_NATIVE, _DENSE or _DENSE_NODE."""
     _check(load().lbm_set_rounding(plan.handle, int(mode)), "lbm_set_rounding")
 
 
@@ -444,11 +444,11 @@ class Solver:
     ``layout``: "dense" (every node stored), "compact" (fluid nodes only,
     ``lbm_compact_bind``), or "auto": compact, which is the faster one at
     every size (a time step of a gradient evaluation on a GB300, dense and
-    compact: D2Q9 FP64 64x32 45.1 and 23.8 us; FP32 301x149 11.0 and 6.8,
-    512x256 10.5 and 7.7, 1024x512 27.3 and 15.5, 4096x2048 392 and 245),
+    compact: D2Q9 FP64 64x32 45.1 and 16.8 us; FP32 301x149 11.0 and 6.6,
+    512x256 10.5 and 7.3, 1024x512 27.3 and 15.5, 4096x2048 392 and 245),
     except on a D2Q9 lattice whose environment or set_kernels() choice asks
     for kernels that only the dense layout has.  The automatic choice rounds
-    as the dense kernels of the lattice do (LBM_ROUND_DENSE).  The
+    as the dense kernels of the lattice do (lbm_set_rounding).  The
     default comes from the LBM_LAYOUT environment variable, else "auto".
     Every array the caller sees is dense either way."""
 
@@ -500,8 +500,8 @@ class Solver:
             self.tables = None  # an open lattice's tables can take more than its solid nodes would
             self.set_layout("dense")
         self._auto_2d = auto and q == 9  # until a layout is named
-        if self._auto_2d and precision == 4 and nx % 2 == 0:  # odd rows: the dense kernels round as the compact ones
-            lbm_set_rounding(p, LBM_ROUND_DENSE)
+        if self._auto_2d and precision == 4:  # odd rows: the dense layout runs one node per thread
+            lbm_set_rounding(p, LBM_ROUND_DENSE if nx % 2 == 0 else LBM_ROUND_DENSE_NODE)
         if self.ws is None:
             self.ws = torch.zeros(lbm_workspace_size(p), dtype=torch.uint8, device=self.device)
 

@@ -131,3 +131,26 @@ def test_the_automatic_layout_rounds_as_the_dense_one(nx, ny):
     s = lbm.Solver(9, nx, ny, precision=4, n_steps=T, geometry=torch.as_tensor(m))
     s.set_kernels(step_family=lbm.LBM_FAMILY_VEC)
     assert s.layout == "dense"
+
+
+# odd rows, and options without a vector or TMA kernel: the dense layout's one-node-per-thread kernels.  tau = 0.73:
+# 1 / tau rounded from FP64 and the quotient of the FP32 numbers differ.
+@pytest.mark.parametrize("nx,ny,option", [(65, 40, None), (301, 149, None), (64, 40, "mrt"), (64, 40, "extrap")])
+def test_the_automatic_layout_is_as_accurate_as_one_node_per_thread(nx, ny, option):
+    m = (np.random.Generator(np.random.PCG64(nx)).uniform(size=(ny, nx)) < 0.2).astype(np.uint8)
+    T, rin, ut = 30, dev(1.0 + W.inlet_profile(ny, seed=5)), dev(W.perturbation((2, ny, nx), seed=6, scale=1e-4))
+    out = []
+    for layout in (None, "dense"):
+        s = lbm.Solver(9, nx, ny, precision=4, n_steps=T, inlet_kind=lbm.LBM_INLET_PROFILE,
+                       geometry=torch.as_tensor(m), layout=layout)
+        if option == "mrt":
+            s.set_collision(lbm.LBM_COLLISION_MRT, 1.1, 1.1, 1.2)
+        elif option == "extrap":
+            lbm.lbm_set_abb_velocity(s.plan, lbm.LBM_ABB_U_EXTRAP)
+        f = s.forward(rin, dev([0.73]), 1.0)
+        _, lam = s.loss_grad(f, ut)
+        out.append((f, *s.adjoint(rin, dev([0.73]), 1.0, lam)))
+    (f, g_in, g_tau), (fd, gd, td) = out
+    assert torch.allclose(f, fd, rtol=0.0, atol=4e-7 * float(fd.abs().max()))  # T steps of contraction differences
+    assert rel(g_in.cpu().numpy(), gd.cpu().numpy()) < 1e-5
+    assert rel(g_tau.cpu().numpy(), td.cpu().numpy()) < 1e-5
