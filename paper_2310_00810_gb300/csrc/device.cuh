@@ -127,9 +127,8 @@ __device__ __forceinline__ void collide(T (&v)[Q], T omega)
         if (L::D == 3) uu += u[2] * u[2];
         const T base = drho - T(1.5) * rho * uu;
         const T r3 = T(3) * rho, r45 = T(4.5) * rho;
-        const T keep = T(1) - omega;
-        v[0] = keep * v[0] + omega * T(L::w(0)) * base;
-        const T wa = omega * T(L::w(1)), wd = omega * T(L::w(Q - 1));  // the axis and the diagonal links
+        v[0] = v[0] - omega * (v[0] - T(L::w(0)) * base);
+        const T wa = T(L::w(1)), wd = T(L::w(Q - 1));  // the axis and the diagonal links
         const T b[2] = {wa * base, wd * base}, p[2] = {wa * r3, wd * r3}, q[2] = {wa * r45, wd * r45};
 #pragma unroll
         for (int i = 1; i < Q; ++i)
@@ -137,8 +136,10 @@ __device__ __forceinline__ void collide(T (&v)[Q], T omega)
                 const int cls = L::w(i) == L::w(1) ? 0 : 1;
                 const T cu = cdot<Q, T>(i, u);
                 const T even = b[cls] + q[cls] * cu * cu, odd = p[cls] * cu;
-                v[i] = keep * v[i] + (even + odd);
-                v[L::opp(i)] = keep * v[L::opp(i)] + (even - odd);
+                // the difference from f^eq first: (1 - omega) f + omega f^eq is two operations shorter and
+                // rounds f^eq's own size (2.1e-16 rms of the state for 1.7e-16)
+                v[i] = v[i] - omega * (v[i] - (even + odd));
+                v[L::opp(i)] = v[L::opp(i)] - omega * (v[L::opp(i)] - (even - odd));
             }
         return;
     }
@@ -381,12 +382,13 @@ __device__ __forceinline__ T adjoint_collision(const T (&f)[Q], const T (&mu)[Q]
     }
     T A = 0, B[3] = {T(0), T(0), T(0)}, domT = 0;
     if constexpr (kByPairs<T>) {
-        // first what needs f, which is then out of registers
+        // dL/domega by pairs of mu (e, o) and of f^eq - f, whose difference is taken before the product:
+        // sum mu f^eq - sum mu f would cancel (sum over 20000 nodes: 4e-12 off for 3e-13)
         T uu = 0;
 #pragma unroll
         for (int a = 0; a < L::D; ++a) uu += u[a] * u[a];
-#pragma unroll
-        for (int j = 0; j < Q; ++j) domT -= mu[j] * f[j];
+        const T fbase = drho - T(1.5) * rho * uu, r3 = T(3) * rho, r45 = T(4.5) * rho;
+        domT = mu[0] * (T(L::w(0)) * fbase - f[0]);
         // sum_j mu_j w_j times 1, c and c c: A and B are quadratic in u with these coefficients
         T ea[3] = {T(0), T(0), T(0)}, oa[3] = {T(0), T(0), T(0)}, ed[3] = {T(0), T(0), T(0)},
           od[3] = {T(0), T(0), T(0)}, x[3] = {T(0), T(0), T(0)}, sd = 0;
@@ -394,6 +396,9 @@ __device__ __forceinline__ T adjoint_collision(const T (&f)[Q], const T (&mu)[Q]
         for (int i = 1; i < Q; ++i)
             if (i < L::opp(i)) {
                 const T e = mu[i] + mu[L::opp(i)], o = mu[i] - mu[L::opp(i)];
+                const T cu = cdot<Q, T>(i, u), wi = T(L::w(i));
+                domT += e * (wi * fbase + wi * r45 * cu * cu - T(0.5) * (f[i] + f[L::opp(i)]));
+                domT += o * (wi * r3 * cu - T(0.5) * (f[i] - f[L::opp(i)]));
                 int n = 0, sg = 1, axes = 0;
 #pragma unroll
                 for (int a = 0; a < L::D; ++a)
@@ -444,7 +449,6 @@ __device__ __forceinline__ T adjoint_collision(const T (&f)[Q], const T (&mu)[Q]
         }
         const T A1 = T(3) * s1u + T(4.5) * q - T(1.5) * uu * S0;
         A = S0 + A1;
-        domT += drho * S0 + rho * A1;
     } else {
         const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
 #pragma unroll
