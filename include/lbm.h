@@ -407,7 +407,9 @@ LBM_API lbm_status lbm_spline_grad(const lbm_plan* plan, int32_t ky, int32_t kz,
  *  d_lambda       lambda^T (plan precision; not modified)
  *  d_grad_rho_in  double[1 or ny nz] out: dL/drho_in
  *  d_grad_tau     double[1] out: dL/dtau
- * Gradient sums are FP64 in a fixed order (deterministic run to run). */
+ * Gradient sums are FP64 in a fixed order (deterministic run to run).
+ * Errors: INVALID_ARG (null pointers, no geometry bound, or the state layout
+ * has changed since the plan's last lbm_forward), UNSUPPORTED, CUDA. */
 LBM_API lbm_status lbm_adjoint(lbm_plan* plan, const double* d_rho_in, const double* d_tau, double rho_out,
                        const void* d_lambda, double* d_grad_rho_in, double* d_grad_tau, void* d_ws, void* stream);
 

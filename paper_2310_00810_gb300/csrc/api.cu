@@ -59,6 +59,7 @@ struct GraphEntry {
 };
 
 constexpr size_t kMaxGraphs = 8;
+constexpr int kSweepLost = -2;  // lbm_plan::fwd_aa: the state layout has changed since the last forward sweep
 
 }  // namespace
 
@@ -73,7 +74,7 @@ struct lbm_plan {
     size_t dense_state_bytes = 0;  // Q N precision: the caller's state arrays
     int dense_n_partial = 0;       // FP64 partial slots of the dense kernels
     void* last_ws = nullptr;
-    int fwd_aa = -1;               // schedule of the last lbm_forward (1: in place): its checkpoints' layouts
+    int fwd_aa = -1;               // schedule of the last lbm_forward (1: in place; -1: none yet; kSweepLost)
     bool use_graphs = true;
     std::vector<GraphEntry> graphs;  // most recently used last
     // second stream and events of the overlapped reverse sweep (created on first use)
@@ -223,6 +224,7 @@ void drop_graphs(lbm_plan* p)
 // Back to the dense layout (a new geometry invalidates the compact tables).
 void set_dense(lbm_plan* p)
 {
+    if (p->info.cmp.nf && p->fwd_aa >= 0) p->fwd_aa = kSweepLost;
     p->info.cmp = Cmp{0, nullptr, nullptr};
     p->info.cmp_map = nullptr;
     p->info.cmp_inst = nullptr;
@@ -581,6 +583,7 @@ lbm_status lbm_compact_bind(lbm_plan* p, int64_t n_fluid, void* d_tables, void* 
     const BCmpInst* inst = nullptr;
     BCmpInst host = {};
     LBM_TRY(compact_build(p->info, n_fluid, d_tables, &c, &cmap, &inst, &host, static_cast<cudaStream_t>(stream)));
+    if (p->info.cmp.nf != c.nf && p->fwd_aa >= 0) p->fwd_aa = kSweepLost;
     p->info.cmp = c;
     p->info.cmp_lat = host.lat;
     p->info.cmp_int = host.n_int;
@@ -619,6 +622,7 @@ lbm_status lbm_forward(lbm_plan* p, const double* d_rho_in, const double* d_tau,
         // one cooperative launch for the whole sweep; g^0 = rest where the sweep expects it
         PersistArgs a = persist_args(p, d_ws);
         a.out = d_f;
+        p->fwd_aa = 0;
         unsigned char* g0 = slot(0) ? slot(0) : ping0;
         if (cudaMemsetAsync(g0, 0, p->info.state_bytes, s) != cudaSuccess) return LBM_ERR_CUDA;
         if (T == 1) return step_launch(p->info, kStreamOnly, g0, d_f, bc, tau, s);
@@ -817,6 +821,8 @@ static lbm_status reverse_sweep(lbm_plan* p, const double* d_rho_in, const doubl
                                 const void* d_lambda, const Window* win, double* d_grad_rho_in, double* d_grad_tau,
                                 void* d_ws, cudaStream_t s)
 {
+    // the checkpoints must come from a forward sweep of the same schedule and state layout
+    if (p->fwd_aa == kSweepLost || (p->fwd_aa >= 0 && p->fwd_aa != (in_place(p) ? 1 : 0))) return LBM_ERR_INVALID_ARG;
     unsigned char* ws = bytes(d_ws);
     p->last_ws = d_ws;
     const double* rho_in = nullptr;
@@ -824,8 +830,6 @@ static lbm_status reverse_sweep(lbm_plan* p, const double* d_rho_in, const doubl
     LBM_TRY(stage_inputs(p, d_ws, d_rho_in, d_tau, &rho_in, &tau, s));
     const Bc bc = make_bc(p, rho_in, rho_out, d_ws);
     const int T = p->desc.n_steps, k = p->k, S = p->S;
-    // the checkpoints must come from a forward sweep of the same schedule (their layouts differ)
-    if (p->fwd_aa >= 0 && p->fwd_aa != (in_place(p) ? 1 : 0)) return LBM_ERR_INVALID_ARG;
     const size_t st = align256(p->info.state_bytes);
     double* grad_acc = reinterpret_cast<double*>(ws + p->ws.grad_acc);
     double* partial = reinterpret_cast<double*>(ws + p->ws.partial);

@@ -195,6 +195,7 @@ class Plan:
         self.N = nx * ny * nz
         self.n_in = ny * nz if inlet_kind == LBM_INLET_PROFILE else 1
         self.dtype = torch.float32 if precision == 4 else torch.float64
+        self._swept = False  # a workspace holds the checkpoints of a forward sweep
 
     @property
     def shape(self):
@@ -335,6 +336,7 @@ def lbm_forward(plan: Plan, rho_in, tau, rho_out: float, f, ws, stream=None) -> 
     _check(load().lbm_forward(plan.handle, _ptr(rho_in, torch.float64, plan.n_in), _ptr(tau, torch.float64, 1),
                               float(rho_out), _ptr(f, plan.dtype, plan.q * plan.N), _ptr(ws, torch.uint8),
                               _stream(stream)), "lbm_forward")
+    plan._swept = True
 
 
 def lbm_step(plan: Plan, rho_in, tau, rho_out: float, f_in, f_out, n_steps: int, ws, stream=None) -> None:
@@ -485,7 +487,8 @@ class Solver:
                                   fill_isolated=False)
             else:
                 lbm_init_geometry(p, self.mask, self.link, self.info, self.porosity, **(geometry or {}))
-        self.layout, self.tables, self.ws = "dense", None, None
+        self._bound, self.tables, self.ws = "dense", None, None
+        self._auto_2d = self._next_dense = False
         layout = layout or os.environ.get("LBM_LAYOUT", "auto")
         if layout not in ("dense", "compact", "auto"):
             raise ValueError(f"layout must be dense, compact or auto, not {layout!r}")
@@ -505,13 +508,24 @@ class Solver:
         if self.ws is None:
             self.ws = torch.zeros(lbm_workspace_size(p), dtype=torch.uint8, device=self.device)
 
+    @property
+    def layout(self) -> str:
+        """The state layout, from the next forward() on."""
+        return "dense" if self._next_dense else self._bound
+
     def set_layout(self, layout: str) -> None:
         """Switches the plan between the dense and the fluid-only state layout
-        (results are the same; the workspace is reallocated)."""
+        (results are the same; the workspace is reallocated, so a reverse sweep
+        needs another forward sweep first).  On a D2Q9 lattice in the automatic
+        layout that holds the checkpoints of a forward sweep, "dense" takes
+        effect at the next forward(): the reverse sweep may still follow."""
         p = self.plan
-        self._auto_2d = False
+        auto, self._auto_2d = self._auto_2d, False
+        self._next_dense = (auto or self._next_dense) and layout == "dense" and p._swept and self._bound == "compact"
+        if self._next_dense:
+            return
         lbm_set_rounding(p, LBM_ROUND_NATIVE)
-        if layout == self.layout:
+        if layout == self._bound:
             return
         if layout == "compact":
             with torch.cuda.device(self.device):
@@ -527,7 +541,7 @@ class Solver:
             self.tables = None
         else:
             raise ValueError(f"layout must be dense or compact, not {layout!r}")
-        self.layout = layout
+        self._bound, p._swept = layout, False
         self.ws = torch.zeros(lbm_workspace_size(p), dtype=torch.uint8, device=self.device)
 
     def run(self, fn):
@@ -569,6 +583,9 @@ class Solver:
 
     def forward(self, rho_in, tau, rho_out, f=None):
         f = self.new_state() if f is None else f
+        if self._next_dense:
+            self._next_dense = False
+            self.set_layout("dense")
         self._fit_ws()
         self.run(lambda: lbm_forward(self.plan, rho_in, tau, rho_out, f, self.ws))
         return f

@@ -1,0 +1,82 @@
+"""The automatic layout of D2Q9 solvers against calls that change it or its kernels."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2310_00810_gb300 import lbm
+from paper_2310_00810_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(x, dtype=torch.float64):
+    return torch.as_tensor(np.ascontiguousarray(x)).to(device="cuda", dtype=dtype)
+
+
+def _mask(nx, ny, seed=2, solid=0.2):
+    m = (np.random.Generator(np.random.PCG64(seed)).uniform(size=(ny, nx)) < solid).astype(np.uint8)
+    m[:, :2] = m[:, -2:] = 0
+    return torch.as_tensor(m)
+
+
+def _solver(nx=64, ny=40, T=30, layout=None, precision=4, **kw):
+    return lbm.Solver(9, nx, ny, precision=precision, n_steps=T, inlet_kind=lbm.LBM_INLET_PROFILE,
+                      geometry=_mask(nx, ny), layout=layout, **kw)
+
+
+def _inputs(s, seed=5):
+    return (dev(1.0 + W.inlet_profile(s.plan.n_in, seed=seed)), dev([0.8]), 1.0), \
+        dev(W.perturbation((2, *s.plan.shape), seed=seed + 1, scale=1e-4))
+
+
+def _gradient(s, between=lambda s: None):
+    p, ut = _inputs(s)
+    f = s.forward(*p)
+    loss, lam = s.loss_grad(f, ut)
+    between(s)
+    return (f, loss, lam, *s.adjoint(*p, lam))
+
+
+def _same(a, b):
+    return all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+# calls that left a default solver's checkpoints alone while its layout was the dense one
+BETWEEN = {
+    "family": lambda s: s.set_kernels(step_family=lbm.LBM_FAMILY_VEC, adjoint_family=lbm.LBM_FAMILY_VEC),
+    "dense": lambda s: s.set_layout("dense"),
+    "two_steps": lambda s: s.set_kernels(steps_per_launch=2),
+    "family_then_step": lambda s: (s.set_kernels(step_family=lbm.LBM_FAMILY_VEC), s.step(*_inputs(s)[0], s.new_state().zero_(), 3)),
+}
+
+
+@pytest.mark.parametrize("precision", [4, 8])
+@pytest.mark.parametrize("between", list(BETWEEN))
+def test_a_layout_named_between_the_sweeps_takes_effect_at_the_next_forward(between, precision):
+    s = _solver(precision=precision)
+    want = _gradient(s)
+    got = _gradient(s, BETWEEN[between])
+    assert torch.count_nonzero(want[3]).item() > 0
+    assert _same(got, want)
+    assert s.layout == "dense"
+    f = s.forward(*_inputs(s)[0])
+    assert s.layout == "dense" and s.tables is None
+    assert torch.allclose(f, want[0], rtol=0.0, atol=1e-6 if precision == 4 else 1e-13)
+
+
+@pytest.mark.parametrize("q,first,second", [(9, "compact", "dense"), (9, "dense", "compact"), (19, "compact", "dense")])
+def test_a_reverse_sweep_after_a_change_of_layout_is_refused(q, first, second):
+    if q == 9:
+        s = _solver(layout=first)
+    else:
+        s = lbm.Solver(19, 20, 12, 9, n_steps=10, inlet_kind=lbm.LBM_INLET_PROFILE, layout=first)
+    p = (dev(1.0 + W.inlet_profile(s.plan.n_in, seed=5)), dev([0.8]), 1.0)
+    f = s.forward(*p)
+    _, lam = s.loss_grad(f, dev(W.perturbation((s.plan.d, *s.plan.shape), seed=6, scale=1e-4)))
+    s.set_layout(second)
+    with pytest.raises(lbm.LBMError) as e:
+        s.adjoint(*p, lam)
+    assert e.value.status == lbm.LBM_ERR_INVALID_ARG
+    s.forward(*p)
+    g_in, _ = s.adjoint(*p, lam)
+    assert torch.count_nonzero(g_in).item() > 0
