@@ -613,9 +613,9 @@ class Solver:
 
     def set_velocity_inlet(self, u) -> None:
         """A velocity inlet u = (ux, uy[, uz]) through x = -1/2 (None: Eq. 6).  It runs in the
-        fluid-only layout, which this switches to."""
+        fluid-only layout, which this names."""
         lbm_set_velocity_inlet(self.plan, u)
-        if u is not None and self.layout != "compact":
+        if u is not None and (self._auto_2d or self.layout != "compact"):
             self.set_layout("compact")
 
     def set_abb_velocity(self, mode: int) -> None:

@@ -80,3 +80,17 @@ def test_a_reverse_sweep_after_a_change_of_layout_is_refused(q, first, second):
     s.forward(*p)
     g_in, _ = s.adjoint(*p, lam)
     assert torch.count_nonzero(g_in).item() > 0
+
+
+@pytest.mark.parametrize("choice", [dict(step_family=lbm.LBM_FAMILY_VEC), dict(persist=1), dict(pdl=0)])
+def test_kernels_after_a_velocity_inlet(choice):
+    """The inlet runs in the fluid-only layout, rounding as that layout named does, whatever is named later."""
+    out = []
+    for layout, kernels in ((None, None), (None, choice), ("compact", None)):
+        s = _solver(layout=layout)
+        s.set_velocity_inlet((0.05, 0.0))
+        if kernels:
+            s.set_kernels(**kernels)
+        assert s.layout == "compact"
+        out.append(_gradient(s))
+    assert _same(out[0], out[1]) and _same(out[0], out[2])
