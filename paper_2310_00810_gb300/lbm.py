@@ -195,7 +195,9 @@ class Plan:
         self.N = nx * ny * nz
         self.n_in = ny * nz if inlet_kind == LBM_INLET_PROFILE else 1
         self.dtype = torch.float32 if precision == 4 else torch.float64
-        self._swept = False  # a workspace holds the checkpoints of a forward sweep
+        self._swept = False   # a workspace holds the checkpoints of a forward sweep
+        self._tables = None   # of the fluid-only layout, while the plan is in it
+        self._resized = True  # the workspace size may have changed since it was last looked up
 
     @property
     def shape(self):
@@ -229,6 +231,7 @@ def lbm_plan_set_kernels(plan: Plan, step_family=LBM_FAMILY_AUTO, adjoint_family
     k = lbm_kernel_choice(step_family, adjoint_family, vec, tma_rows, pdl, persist, overlap, adjoint_tma_rows,
                           steps_per_launch, recompute_family, aa)
     _check(load().lbm_plan_set_kernels(plan.handle, C.byref(k)), "lbm_plan_set_kernels")
+    plan._resized = True
 
 
 def lbm_plan_get_kernels(plan: Plan) -> dict:
@@ -253,11 +256,18 @@ def lbm_init_geometry(plan: Plan, mask, link, info, porosity=None, kind=LBM_GEOM
                                     _ptr(info, torch.int64, 4), _stream(stream)), "lbm_init_geometry")
     plan._link = link  # keep the bound geometry alive with the plan
     plan._mask = mask
+    _geometry_bound(plan)
 
 
 def lbm_bind_geometry(plan: Plan, link) -> None:
     _check(load().lbm_bind_geometry(plan.handle, _ptr(link, torch.int32, plan.N)), "lbm_bind_geometry")
     plan._link = link
+    _geometry_bound(plan)
+
+
+def _geometry_bound(plan: Plan) -> None:
+    if plan._tables is not None:  # the fluid-only tables are of the geometry before: the plan is dense again
+        plan._tables, plan._swept, plan._resized = None, False, True
 
 
 def lbm_compact_size(plan: Plan, n_fluid: int) -> int:
@@ -269,7 +279,8 @@ def lbm_compact_size(plan: Plan, n_fluid: int) -> int:
 def lbm_compact_bind(plan: Plan, n_fluid: int, tables, stream=None) -> None:
     _check(load().lbm_compact_bind(plan.handle, int(n_fluid), _ptr(tables, torch.uint8), _stream(stream)),
            "lbm_compact_bind")
-    plan._tables = tables  # the plan reads the tables while it is bound to them
+    # the plan reads the tables while it is bound to them
+    plan._tables, plan._resized = (tables if n_fluid else None), True
 
 
 def lbm_set_abb_velocity(plan: Plan, mode: int) -> None:
@@ -487,7 +498,7 @@ class Solver:
                                   fill_isolated=False)
             else:
                 lbm_init_geometry(p, self.mask, self.link, self.info, self.porosity, **(geometry or {}))
-        self._bound, self.tables, self.ws = "dense", None, None
+        self._ws = None
         self._auto_2d = self._next_dense = False
         layout = layout or os.environ.get("LBM_LAYOUT", "auto")
         if layout not in ("dense", "compact", "auto"):
@@ -500,13 +511,35 @@ class Solver:
         except torch.cuda.OutOfMemoryError:
             if not (auto and q == 9):
                 raise
-            self.tables = None  # an open lattice's tables can take more than its solid nodes would
+            # an open lattice's tables can take more than its solid nodes would
             self.set_layout("dense")
         self._auto_2d = auto and q == 9  # until a layout is named
         if self._auto_2d and precision == 4:  # odd rows: the dense layout runs one node per thread
             lbm_set_rounding(p, LBM_ROUND_DENSE if nx % 2 == 0 else LBM_ROUND_DENSE_NODE)
-        if self.ws is None:
-            self.ws = torch.zeros(lbm_workspace_size(p), dtype=torch.uint8, device=self.device)
+        _ = self.ws  # allocated here, not in the first sweep
+
+    @property
+    def ws(self) -> torch.Tensor:
+        """The workspace, grown where the plan has come to need more: another geometry moves it to the dense
+        layout, and clearing the in-place schedule (aa) takes two states."""
+        if self.plan._resized:
+            need = lbm_workspace_size(self.plan)
+            if self._ws is None or need > self._ws.numel():
+                self._ws = torch.zeros(need, dtype=torch.uint8, device=self.device)
+            self.plan._resized = False
+        return self._ws
+
+    @ws.setter
+    def ws(self, t) -> None:
+        self._ws, self.plan._resized = t, True
+
+    @property
+    def tables(self):
+        return self.plan._tables
+
+    @property
+    def _bound(self) -> str:
+        return "dense" if self.plan._tables is None else "compact"
 
     @property
     def layout(self) -> str:
@@ -530,18 +563,20 @@ class Solver:
         if layout == "compact":
             with torch.cuda.device(self.device):
                 torch.cuda.current_stream().synchronize()
-            nf = int(self.info[3].item()) if self.info is not None else int((self.link[: p.N] >= 0).sum().item())
+            if self.info is not None and p._link is self.link:
+                nf = int(self.info[3].item())
+            else:
+                nf = int((p._link[: p.N] >= 0).sum().item())
             if nf == 0:
                 return  # nothing to compact: an all-solid lattice stays dense
             tables = torch.empty(max(lbm_compact_size(p, nf), 256), dtype=torch.uint8, device=self.device)
             self.run(lambda: lbm_compact_bind(p, nf, tables, self.stream))
-            self.tables, self.n_fluid = tables, nf
+            self.n_fluid = nf
         elif layout == "dense":
             self.run(lambda: lbm_compact_bind(p, 0, None, self.stream))
-            self.tables = None
         else:
             raise ValueError(f"layout must be dense or compact, not {layout!r}")
-        self._bound, p._swept = layout, False
+        p._swept = False
         self.ws = torch.zeros(lbm_workspace_size(p), dtype=torch.uint8, device=self.device)
 
     def run(self, fn):
@@ -573,27 +608,20 @@ class Solver:
         if self._auto_2d and self._DENSE_CHOICE.intersection(choice):
             self.set_layout("dense")
         lbm_plan_set_kernels(self.plan, **choice)
-        self._fit_ws()
-
-    def _fit_ws(self) -> None:
-        # clearing the in-place schedule (aa) after the workspace was sized for it grows the need by two states
-        need = lbm_workspace_size(self.plan)
-        if need > self.ws.numel():
-            self.ws = torch.zeros(need, dtype=torch.uint8, device=self.device)
 
     def forward(self, rho_in, tau, rho_out, f=None):
         f = self.new_state() if f is None else f
         if self._next_dense:
             self._next_dense = False
             self.set_layout("dense")
-        self._fit_ws()
-        self.run(lambda: lbm_forward(self.plan, rho_in, tau, rho_out, f, self.ws))
+        ws = self.ws
+        self.run(lambda: lbm_forward(self.plan, rho_in, tau, rho_out, f, ws))
         return f
 
     def step(self, rho_in, tau, rho_out, f_in, n_steps, f_out=None):
         f_out = torch.empty_like(f_in) if f_out is None else f_out
-        self._fit_ws()
-        self.run(lambda: lbm_step(self.plan, rho_in, tau, rho_out, f_in, f_out, n_steps, self.ws))
+        ws = self.ws
+        self.run(lambda: lbm_step(self.plan, rho_in, tau, rho_out, f_in, f_out, n_steps, ws))
         return f_out
 
     def loss_grad(self, f, u_target, roi=None, loss=None, lam=None):

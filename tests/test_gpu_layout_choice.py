@@ -94,3 +94,18 @@ def test_kernels_after_a_velocity_inlet(choice):
         assert s.layout == "compact"
         out.append(_gradient(s))
     assert _same(out[0], out[1]) and _same(out[0], out[2])
+
+
+def test_another_geometry_moves_the_solver_to_the_dense_layout():
+    s = _solver()
+    m = _mask(64, 40, seed=9).cuda()
+    s.mask[: s.plan.N].copy_(m.reshape(-1))
+    lbm.lbm_init_geometry(s.plan, s.mask, s.link, s.info, s.porosity, kind=lbm.LBM_GEOM_MASK, fill_isolated=False)
+    # the plan is dense from here on; a sweep through s.ws must find room for it
+    assert s.layout == "dense"
+    assert s.ws.numel() >= lbm.lbm_workspace_size(s.plan)
+    fresh = lbm.Solver(9, 64, 40, n_steps=30, inlet_kind=lbm.LBM_INLET_PROFILE, geometry=m, layout="dense")
+    assert _same(_gradient(s), _gradient(fresh))
+    s.set_velocity_inlet((0.05, 0.0))
+    assert s.layout == "compact"
+    assert torch.isfinite(s.forward(*_inputs(s)[0])).all()
