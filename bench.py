@@ -799,7 +799,7 @@ def kernel_rooflines(device, hbm_peak, name, n_launch, layout=None, aa=0):
     wl = W.WORKLOADS[name]
     s = lbm.Solver(wl.q, wl.nx, wl.ny, wl.nz, precision=wl.precision, n_steps=n_launch, ckpt_stride=n_launch,
                    geometry=dict(kind=wl.geom_kind, seed=wl.seed, r_min=wl.r_min, r_max=wl.r_max,
-                                 target_porosity=wl.porosity), device=device, layout=layout)
+                                 target_porosity=wl.porosity), device=device, layout=layout or ("compact" if aa else None))
     nf, N, q, sz = int(s.info[3].item()), wl.nodes, wl.q, wl.precision
     if aa:
         s.set_kernels(**dict(lbm.lbm_plan_get_kernels(s.plan), aa=1))

@@ -197,6 +197,7 @@ class Plan:
         self.dtype = torch.float32 if precision == 4 else torch.float64
         self._swept = False   # a workspace holds the checkpoints of a forward sweep
         self._tables = None   # of the fluid-only layout, while the plan is in it
+        self._ignores_aa = False
         self._resized = True  # the workspace size may have changed since it was last looked up
 
     @property
@@ -228,6 +229,8 @@ def lbm_plan_destroy(plan: Plan) -> None:
 def lbm_plan_set_kernels(plan: Plan, step_family=LBM_FAMILY_AUTO, adjoint_family=LBM_FAMILY_AUTO, vec=4,
                          tma_rows=8, pdl=1, persist=0, overlap=1, adjoint_tma_rows=0, steps_per_launch=1,
                          aa=0, recompute_family=LBM_FAMILY_AUTO) -> None:
+    if plan._ignores_aa:  # the automatic D2Q9 layout of a Solver
+        aa = 0
     k = lbm_kernel_choice(step_family, adjoint_family, vec, tma_rows, pdl, persist, overlap, adjoint_tma_rows,
                           steps_per_launch, recompute_family, aa)
     _check(load().lbm_plan_set_kernels(plan.handle, C.byref(k)), "lbm_plan_set_kernels")
@@ -461,7 +464,8 @@ class Solver:
     512x256 10.5 and 7.3, 1024x512 27.3 and 15.5, 4096x2048 392 and 245),
     except on a D2Q9 lattice whose environment or set_kernels() choice asks
     for kernels that only the dense layout has.  The automatic choice rounds
-    as the dense kernels of the lattice do (lbm_set_rounding).  The
+    as the dense kernels of the lattice do (lbm_set_rounding), and on D2Q9
+    ignores the in-place schedule (aa), as the dense layout does.  The
     default comes from the LBM_LAYOUT environment variable, else "auto".
     Every array the caller sees is dense either way."""
 
@@ -513,7 +517,7 @@ class Solver:
                 raise
             # an open lattice's tables can take more than its solid nodes would
             self.set_layout("dense")
-        self._auto_2d = auto and q == 9  # until a layout is named
+        self._auto_2d = p._ignores_aa = auto and q == 9  # until a layout is named
         if self._auto_2d and precision == 4:  # odd rows: the dense layout runs one node per thread
             lbm_set_rounding(p, LBM_ROUND_DENSE if nx % 2 == 0 else LBM_ROUND_DENSE_NODE)
         _ = self.ws  # allocated here, not in the first sweep
@@ -555,6 +559,7 @@ class Solver:
         p = self.plan
         auto, self._auto_2d = self._auto_2d, False
         self._next_dense = (auto or self._next_dense) and layout == "dense" and p._swept and self._bound == "compact"
+        p._ignores_aa = self._next_dense
         if self._next_dense:
             return
         lbm_set_rounding(p, LBM_ROUND_NATIVE)

@@ -109,3 +109,20 @@ def test_another_geometry_moves_the_solver_to_the_dense_layout():
     s.set_velocity_inlet((0.05, 0.0))
     assert s.layout == "compact"
     assert torch.isfinite(s.forward(*_inputs(s)[0])).all()
+
+
+@pytest.mark.parametrize("first", ["aa", "extrap"])
+def test_in_place_streaming_on_the_automatic_layout(first):
+    """It is ignored there, as it was while the dense layout was the automatic one."""
+    want = _solver()
+    lbm.lbm_set_abb_velocity(want.plan, lbm.LBM_ABB_U_EXTRAP)
+    s = _solver()
+    for name in ("aa", "extrap") if first == "aa" else ("extrap", "aa"):
+        if name == "aa":
+            s.set_kernels(aa=1)
+        else:
+            s.set_abb_velocity(lbm.LBM_ABB_U_EXTRAP)
+    assert _same(_gradient(s), _gradient(want))
+    s = _solver()
+    want = _gradient(s)
+    assert _same(_gradient(s, lambda s: s.set_kernels(aa=1)), want)
