@@ -471,8 +471,10 @@ class Solver:
 
     _DENSE_ENV = ("LBM_KERNEL", "LBM_VEC", "LBM_TMA", "LBM_TMA_MIN_TILES", "LBM_TMA_VARIANT", "LBM_TMA_ROWS",
                   "LBM_TMA_WAVES", "LBM_STEP_VARIANT", "LBM_PERSIST")
-    _DENSE_CHOICE = {"step_family", "adjoint_family", "vec", "tma_rows", "persist", "adjoint_tma_rows",
-                     "steps_per_launch", "recompute_family"}
+    # what an automatic choice leaves of the dense layout's kernels (lbm_plan_set_kernels)
+    _DENSE_CHOICE = dict(step_family=(LBM_FAMILY_AUTO,), adjoint_family=(LBM_FAMILY_AUTO,),
+                         recompute_family=(LBM_FAMILY_AUTO,), vec=(4,), tma_rows=(8,), adjoint_tma_rows=(0, 8),
+                         persist=(0,), steps_per_launch=(0, 1))
 
     def __init__(self, q, nx, ny, nz=1, precision=4, n_steps=1, ckpt_stride=0, loss_kind=LBM_LOSS_VEC,
                  loss_norm=LBM_NORM_SUM, inlet_kind=LBM_INLET_CONST, geometry=None, device="cuda", link=None,
@@ -609,10 +611,11 @@ class Solver:
 
     def set_kernels(self, **choice) -> None:
         """lbm_plan_set_kernels, then a larger workspace where the choice needs one.  On a D2Q9 lattice in
-        the automatic layout, naming a kernel family of the dense layout switches to that layout."""
-        if self._auto_2d and self._DENSE_CHOICE.intersection(choice):
-            self.set_layout("dense")
+        the automatic layout, a choice among the dense layout's kernels (another value than _DENSE_CHOICE
+        has) switches to that layout."""
         lbm_plan_set_kernels(self.plan, **choice)
+        if self._auto_2d and any(choice.get(k, v[0]) not in v for k, v in self._DENSE_CHOICE.items()):
+            self.set_layout("dense")
 
     def forward(self, rho_in, tau, rho_out, f=None):
         f = self.new_state() if f is None else f

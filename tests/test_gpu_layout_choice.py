@@ -126,3 +126,13 @@ def test_in_place_streaming_on_the_automatic_layout(first):
     s = _solver()
     want = _gradient(s)
     assert _same(_gradient(s, lambda s: s.set_kernels(aa=1)), want)
+
+
+def test_only_another_dense_choice_leaves_the_automatic_layout():
+    s = _solver()
+    for choice in (dict(persist=0), dict(vec=4, tma_rows=8), dict(steps_per_launch=1), dict(adjoint_tma_rows=0),
+                   dict(step_family=lbm.LBM_FAMILY_AUTO, pdl=0), lbm.lbm_plan_get_kernels(s.plan)):
+        s.set_kernels(**choice)
+        assert s.layout == "compact", choice
+    s.set_kernels(recompute_family=lbm.LBM_FAMILY_VEC)
+    assert s.layout == "dense"
