@@ -136,3 +136,17 @@ def test_only_another_dense_choice_leaves_the_automatic_layout():
         assert s.layout == "compact", choice
     s.set_kernels(recompute_family=lbm.LBM_FAMILY_VEC)
     assert s.layout == "dense"
+
+
+# rows that the one-node-per-thread kernels take where the TMA or register kernels apply too
+@pytest.mark.parametrize("nx,ny", [(64, 40), (66, 40), (512, 128)])
+def test_the_dense_layouts_kernel_families_round_alike(nx, ny):
+    out = []
+    for family in (lbm.LBM_FAMILY_AUTO, lbm.LBM_FAMILY_VEC):
+        s = _solver(nx, ny, layout="dense")
+        lbm.lbm_plan_set_kernels(s.plan, step_family=family, adjoint_family=family)
+        out.append(_gradient(s))
+    (f, _, lam, g_in, g_tau), (fv, _, lamv, gv, tv) = out
+    assert torch.equal(f, fv) and torch.equal(lam, lamv)
+    # FP32 adjoint states of other compilations, FP32 warp sums over other groups of nodes
+    assert ((g_in - gv).norm() / gv.norm()).item() < 1e-6 and abs((g_tau - tv) / tv).item() < 1e-5
