@@ -8,11 +8,15 @@ on/off and the one-launch persistent sweeps, the overlapped reverse sweep (recom
 the segment recompute on a register family beside the adjoint, two stream-collide steps per launch
 (D2Q9 FP32), then the fluid-only (compact) layout with two-buffer or in-place streaming, and keeps the
 fastest.  Only the speed differs between candidates;
-every family and layout computes the same step.  Results are cached in JSON
-keyed by GPU name, Q, precision, lattice size and inlet kind.
+every family and layout computes the same step, and a solver whose layout was
+automatic keeps its rounding (lbm_set_rounding).  Results are cached in JSON
+keyed by GPU name, the kernels' sources, Q, precision, lattice size, inlet
+kind, collision, Eq. 6 velocity and porosity (in steps of 5 %: the fluid-only
+layout's time goes by fluid nodes).
 
-Timing uses a short tuning plan bound to the solver's geometry (T_tune time
-steps), with CUDA events around graph-replayed launch sequences.
+Timing uses a short tuning plan bound to the solver's geometry with its
+collision and Eq. 6 velocity (T_tune time steps), with CUDA events around
+graph-replayed launch sequences.
 
 ``tune_batch`` does the same for a batch of lattices (lbm.Batch): it times a
 whole gradient evaluation (forward, loss, checkpointed adjoint) of a short
@@ -22,6 +26,9 @@ layout, and keeps the faster.
 """
 from __future__ import annotations
 
+import functools
+import glob
+import hashlib
 import json
 import os
 import threading
@@ -34,9 +41,25 @@ _lock = threading.Lock()
 DEFAULT_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune.json")
 
 
-def _key(p: lbm.Plan) -> str:
-    name = torch.cuda.get_device_name(torch.cuda.current_device()).replace(" ", "_")
-    return f"{name}|q{p.q}|p{p.precision}|{p.nx}x{p.ny}x{p.nz}|{p.inlet_kind}"
+@functools.lru_cache(maxsize=None)
+def _sources() -> str:
+    """A digest of the kernels' sources: a measurement is of one version of them."""
+    h = hashlib.sha1()
+    for path in sorted(glob.glob(os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc", "*"))):
+        with open(path, "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:12]
+
+
+def _gpu() -> str:
+    return torch.cuda.get_device_name(torch.cuda.current_device()).replace(" ", "_") + "|" + _sources()
+
+
+def _key(solver: lbm.Solver) -> str:
+    p = solver.plan
+    fluid = int((p._link[: p.N] >= 0).sum().item()) / p.N
+    return (f"{_gpu()}|q{p.q}|p{p.precision}|{p.nx}x{p.ny}x{p.nz}|{p.inlet_kind}|c{lbm.lbm_get_collision(p)[0]}"
+            f"|u{lbm.lbm_get_abb_velocity(p)}|f{round(20 * fluid)}")
 
 
 def _load(path):
@@ -96,7 +119,7 @@ def tune(solver: lbm.Solver, t_tune: int = 64, repeats: int = 3, cache: str | No
         # periodic link words wrap in y, which only the fluid-only kernels follow: no dense candidates
         return {"choice": lbm.lbm_plan_get_kernels(p), "layout": solver.layout, "timings_us": {},
                 "us_per_time_step": None, "skipped": "periodic y runs in the fluid-only layout only"}
-    key = _key(p)
+    key = _key(solver)
     if use_cache and cache:
         hit = _load(cache).get(key)
         if hit:
@@ -107,6 +130,9 @@ def tune(solver: lbm.Solver, t_tune: int = 64, repeats: int = 3, cache: str | No
     tp = lbm.Solver(p.q, p.nx, p.ny, p.nz, precision=p.precision, n_steps=t_tune, ckpt_stride=8,
                     inlet_kind=p.inlet_kind, link=solver.link, mask=solver.mask, device=dev, layout="dense")
     tq = tp.plan
+    mode, rates = lbm.lbm_get_collision(p)
+    lbm.lbm_set_collision(tq, mode, *rates)
+    lbm.lbm_set_abb_velocity(tq, lbm.lbm_get_abb_velocity(p))
     rho_in = torch.full((tq.n_in,), 1.001, dtype=torch.float64, device=dev)
     tau = torch.tensor([0.8], dtype=torch.float64, device=dev)
     a = tp.new_state().zero_()
@@ -188,6 +214,7 @@ def tune(solver: lbm.Solver, t_tune: int = 64, repeats: int = 3, cache: str | No
                 best, best_t = c, t
     layout = "dense"
     tp.set_layout("compact")
+    lbm.lbm_set_rounding(tq, p._rounding)
     if tp.layout == "compact":
         for pdl in (1, 0):
             c = dict(best, pdl=pdl, persist=0, overlap=1, steps_per_launch=1, aa=0)
@@ -219,7 +246,10 @@ def solver_uw_extrap(solver: lbm.Solver) -> bool:
 
 
 def _apply(solver: lbm.Solver, result: dict) -> None:
+    rounding = solver.plan._rounding
     solver.set_layout(result.get("layout", "dense"))
+    if solver.layout == "compact":
+        lbm.lbm_set_rounding(solver.plan, rounding)
     choice = dict(result["choice"])
     if solver_uw_extrap(solver):
         choice["aa"] = 0
@@ -227,11 +257,8 @@ def _apply(solver: lbm.Solver, result: dict) -> None:
 
 
 def _batch_key(b) -> str:
-    import hashlib
-
-    name = torch.cuda.get_device_name(torch.cuda.current_device()).replace(" ", "_")
     geo = hashlib.sha1(repr((b.sizes, b.geometries)).encode()).hexdigest()[:16]
-    return f"{name}|batch|q{b.q}|p{b.precision}|n{b.n}|{geo}|{b.inlet_kind}"
+    return f"{_gpu()}|batch|q{b.q}|p{b.precision}|n{b.n}|{geo}|{b.inlet_kind}"
 
 
 def tune_batch(batch, t_tune: int = 64, repeats: int = 2, cache: str | None = DEFAULT_CACHE, use_cache: bool = True,

@@ -198,6 +198,7 @@ class Plan:
         self._swept = False   # a workspace holds the checkpoints of a forward sweep
         self._tables = None   # of the fluid-only layout, while the plan is in it
         self._ignores_aa = False
+        self._rounding = LBM_ROUND_NATIVE
         self._resized = True  # the workspace size may have changed since it was last looked up
 
     @property
@@ -304,6 +305,7 @@ def lbm_set_collision(plan: Plan, mode: int, s_e: float = 1.0, s_eps: float = 1.
 def lbm_set_rounding(plan: Plan, mode: int) -> None:
     """How the fluid-only layout's D2Q9 FP32 kernels round: LBM_ROUND_NATIVE, _DENSE or _DENSE_NODE."""
     _check(load().lbm_set_rounding(plan.handle, int(mode)), "lbm_set_rounding")
+    plan._rounding = int(mode)
 
 
 def lbm_set_periodic_y(plan: Plan, on: bool) -> None:

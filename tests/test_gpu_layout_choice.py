@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2310_00810_gb300 import autotune
 from paper_2310_00810_gb300 import lbm
 from paper_2310_00810_gb300 import workloads as W
 
@@ -25,7 +26,7 @@ def _solver(nx=64, ny=40, T=30, layout=None, precision=4, **kw):
 
 
 def _inputs(s, seed=5):
-    return (dev(1.0 + W.inlet_profile(s.plan.n_in, seed=seed)), dev([0.8]), 1.0), \
+    return (dev(1.0 + W.inlet_profile(s.plan.n_in, seed=seed)), dev([0.73]), 1.0), \
         dev(W.perturbation((2, *s.plan.shape), seed=seed + 1, scale=1e-4))
 
 
@@ -150,3 +151,25 @@ def test_the_dense_layouts_kernel_families_round_alike(nx, ny):
     assert torch.equal(f, fv) and torch.equal(lam, lamv)
     # FP32 adjoint states of other compilations, FP32 warp sums over other groups of nodes
     assert ((g_in - gv).norm() / gv.norm()).item() < 1e-6 and abs((g_tau - tv) / tv).item() < 1e-5
+
+
+# tau = 0.73: 1 / tau rounded from FP64 and the quotient of the FP32 numbers differ
+@pytest.mark.parametrize("nx", [64, 65])
+def test_tuning_keeps_the_rounding_of_the_automatic_layout(nx):
+    s = _solver(nx, 41)
+    before = _gradient(s)
+    autotune._apply(s, dict(layout="compact", choice=dict(pdl=1, overlap=0, aa=1)))
+    assert s.layout == "compact" and lbm.lbm_plan_get_kernels(s.plan)["aa"] == 1
+    assert _same(_gradient(s), before)
+
+
+def test_tuning_results_are_kept_apart_by_what_decides_them(tmp_path):
+    cache = str(tmp_path / "t.json")
+    s = _solver(65, 41)
+    autotune.tune(s, t_tune=8, repeats=1, cache=cache)
+    assert autotune.tune(s, t_tune=8, repeats=1, cache=cache)["cached"]
+    mrt = _solver(65, 41)
+    mrt.set_collision(lbm.LBM_COLLISION_MRT, 1.1, 1.1, 1.2)
+    assert not autotune.tune(mrt, t_tune=8, repeats=1, cache=cache)["cached"]
+    opened = lbm.Solver(9, 65, 41, n_steps=30, inlet_kind=lbm.LBM_INLET_PROFILE, geometry=_mask(65, 41, solid=0.0))
+    assert not autotune.tune(opened, t_tune=8, repeats=1, cache=cache)["cached"]
