@@ -533,12 +533,16 @@ class Solver:
         if self.plan._resized:
             need = lbm_workspace_size(self.plan)
             if self._ws is None or need > self._ws.numel():
-                self._ws = torch.zeros(need, dtype=torch.uint8, device=self.device)
+                self.ws = torch.zeros(need, dtype=torch.uint8, device=self.device)
             self.plan._resized = False
         return self._ws
 
     @ws.setter
     def ws(self, t) -> None:
+        # calls made straight on the solver's stream may still use the old one, and wait for nothing of the new one
+        if self._ws is not None:
+            self._ws.record_stream(self.stream)
+        self.stream.wait_stream(torch.cuda.current_stream(self.device))
         self._ws, self.plan._resized = t, True
 
     @property
