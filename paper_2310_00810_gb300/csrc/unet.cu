@@ -697,6 +697,16 @@ constexpr unsigned kUmmaTimeout = 1u;
 constexpr uint64_t kUmmaWaitNs = 500000000ull;  // 0.5 s per wait (a copy or an MMA step takes microseconds)
 constexpr int kUmmaStages = 4;  // weight gradients
 
+// Whether a wait of an earlier launch gave up (the flag is not yet read by
+// unet_get_status): the launch then does nothing, so that one failure costs one
+// wait limit, not one per CTA.  One thread reads the word for the block: the
+// launch before may set it at any time until pdl_enter, and threads that saw
+// different values would part before the warp-wide tensor-memory allocation.
+__device__ __forceinline__ bool umma_gave_up()
+{
+    return __syncthreads_or(threadIdx.x == 0 && *reinterpret_cast<volatile unsigned*>(&g_umma_status) != 0u) != 0;
+}
+
 // Stages of the convolution kernel's ring.  A tile has 9 to 36 steps, a fill
 // latency before them and an epilogue after, none of which overlap inside a
 // CTA, so what keeps an SM busy on a large grid is several CTAs on it: few
@@ -726,9 +736,7 @@ __global__ void __launch_bounds__(128, 1) k_umma_conv(const __grid_constant__ CU
     using SM = UmmaSmem<KC, BN, DEPTH>;
     constexpr int kStages = SM::STAGES;
     namespace U = umma;
-    // a wait of an earlier launch gave up (flag not yet read by unet_get_status): do nothing, so that one
-    // failure costs one wait limit, not one per CTA
-    if (*reinterpret_cast<volatile unsigned*>(&g_umma_status)) {
+    if (umma_gave_up()) {
         pdl_enter();
         return;
     }
@@ -885,7 +893,7 @@ __global__ void __launch_bounds__(128, 1) k_umma_wgrad(const __grid_constant__ C
     using WS = WgradSmem<AW, BN, BW>;
     constexpr int A_BYTES = WS::A_BYTES, STAGE = WS::STAGE;
     namespace U = umma;
-    if (*reinterpret_cast<volatile unsigned*>(&g_umma_status)) {
+    if (umma_gave_up()) {
         pdl_enter();
         return;
     }
