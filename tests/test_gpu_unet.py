@@ -178,3 +178,22 @@ def test_trained_network_beats_the_zero_start():
     assert all(r["unet"]["converged"] for r in rows)
     assert np.mean([r["unet"]["gradient_evaluations"] for r in rows]) < np.mean(
         [r["zero"]["gradient_evaluations"] for r in rows])
+
+
+# What the grid of a convolution decides, at sizes on both sides of one and two CTAs per SM: eight, four or fewer
+# ring stages and tiles of 32 to 256 columns; and the input layer's kernels where a block takes several strips,
+# rows of more than one strip, a last strip of 16 or 32 pixels.
+@pytest.mark.parametrize("base,H,W,B", [(32, 128, 256, 1), (32, 128, 256, 2), (32, 128, 256, 4), (32, 128, 256, 20),
+                                        (64, 64, 128, 8), (64, 128, 128, 12), (32, 16, 272, 24), (32, 16, 288, 40)])
+def test_grids_and_strips_agree_with_mma_sync(base, H, W, B, _engine_restored):
+    res = {}
+    for eng in (N.ENGINE_MMA_SYNC, N.ENGINE_TCGEN05):
+        N.unet_set_engine(eng)
+        net, x, target, loss, out, grads = gpu_case(base, H, W, B, seed=31)
+        res[eng] = (loss, out, grads)
+    assert N.unet_get_status() == lbm.LBM_OK
+    (l0, o0, g0), (l1, o1, g1) = res[N.ENGINE_MMA_SYNC], res[N.ENGINE_TCGEN05]
+    assert rel(o1, o0) < 1e-2 and abs(l1 - l0) <= 1e-2 * abs(l0)
+    assert rel(np.concatenate(g1), np.concatenate(g0)) < 3e-2
+    for a, b in zip(g1, g0):
+        assert rel(a, b) < 0.1

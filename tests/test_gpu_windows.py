@@ -154,3 +154,66 @@ def test_the_automatic_layout_is_as_accurate_as_one_node_per_thread(nx, ny, opti
     assert torch.allclose(f, fd, rtol=0.0, atol=4e-7 * float(fd.abs().max()))  # T steps of contraction differences
     assert rel(g_in.cpu().numpy(), gd.cpu().numpy()) < 1e-5
     assert rel(g_tau.cpu().numpy(), td.cpu().numpy()) < 1e-5
+
+
+def _default_and_dense(nx, ny, option, T=5):
+    """(state, seed, dL/drho_in, dL/dtau) of the automatic layout and of the dense layout's register (even rows)
+    or one-node-per-thread kernels (odd rows, or an option that only they have)."""
+    m = (np.random.Generator(np.random.PCG64(nx)).uniform(size=(ny, nx)) < 0.25).astype(np.uint8)
+    rin, ut = dev(1.0 + W.inlet_profile(ny, seed=5)), dev(W.perturbation((2, ny, nx), seed=6, scale=1e-4))
+    out = []
+    for layout in (None, "dense"):
+        s = lbm.Solver(9, nx, ny, precision=4, n_steps=T, inlet_kind=lbm.LBM_INLET_PROFILE,
+                       geometry=torch.as_tensor(m), layout=layout)
+        assert int(s.info[3].item()) > 600000
+        if option == "mrt":
+            s.set_collision(lbm.LBM_COLLISION_MRT, 1.1, 1.1, 1.2)
+        elif option == "extrap":
+            s.set_abb_velocity(lbm.LBM_ABB_U_EXTRAP)
+        if layout:
+            family = lbm.LBM_FAMILY_VEC if nx % 2 == 0 else lbm.LBM_FAMILY_SCALAR
+            lbm.lbm_plan_set_kernels(s.plan, step_family=family, adjoint_family=family)
+        else:
+            assert s.layout == "compact"
+        f = s.forward(rin, dev([0.73]), 1.0)
+        _, lam = s.loss_grad(f, ut)
+        out.append((f, lam, *s.adjoint(rin, dev([0.73]), 1.0, lam)))
+    return out
+
+
+# past the pipelined kernels' threshold, in the rounding of the automatic layout
+@pytest.mark.parametrize("nx,ny,option", [(1000, 830, None), (1001, 831, None), (1000, 830, "mrt"),
+                                          (1001, 831, "mrt"), (1000, 830, "extrap"), (1001, 831, "extrap")])
+def test_the_automatic_layout_past_the_pipelined_threshold(nx, ny, option):
+    (f, lam, g_in, g_tau), (fd, lamd, gd, td) = _default_and_dense(nx, ny, option)
+    if option is None and nx % 2 == 0:
+        assert torch.equal(f, fd) and torch.equal(lam, lamd)
+    else:
+        assert torch.allclose(f, fd, rtol=0.0, atol=4e-7 * float(fd.abs().max()))  # contraction differences
+    assert rel(g_in.cpu().numpy(), gd.cpu().numpy()) < 1e-5
+    assert rel(g_tau.cpu().numpy(), td.cpu().numpy()) < 1e-5
+
+
+@pytest.mark.parametrize("mrt", [False, True])
+def test_a_periodic_lattice_repeated_past_the_pipelined_threshold(mrt):
+    """A lattice periodic in y with a ramped velocity inlet, and nine copies of it one above the other: the same
+    flow, by one node per thread and by the pipelined kernels."""
+    nx, ny, copies, T = 1000, 90, 9, 6
+    m = (np.random.Generator(np.random.PCG64(8)).uniform(size=(ny, nx)) < 0.2).astype(np.uint8)
+    ut = W.perturbation((2, 2, ny, nx), seed=9, scale=1e-3)
+    out = []
+    for n in (1, copies):
+        s = lbm.Solver(9, nx, n * ny, precision=4, n_steps=T, geometry=torch.as_tensor(np.tile(m, (n, 1))),
+                       periodic_y=True)
+        assert (int(s.info[3].item()) > 600000) == (n == copies)
+        s.set_velocity_inlet((0.05, 0.01))
+        s.set_velocity_ramp(4)
+        if mrt:
+            s.set_collision(lbm.LBM_COLLISION_MRT, 1.1, 1.1, 1.2)
+        f = s.forward(dev([1.0]), dev([0.73]), 1.0)
+        L, _, g = s.adjoint_window(dev([1.0]), dev([0.73]), 1.0, f, [3, T], dev(np.tile(ut, (1, 1, n, 1))))
+        out.append((f.cpu().numpy(), L.item(), g.item()))
+    (f1, L1, g1), (fn, Ln, gn) = out
+    # the same operations per node, of two compilations
+    assert np.abs(fn - np.tile(f1, (1, copies, 1))).max() <= 4e-7 * np.abs(f1).max()
+    assert abs(Ln - copies * L1) <= 1e-5 * abs(Ln) and abs(gn - copies * g1) <= 1e-4 * abs(gn)
