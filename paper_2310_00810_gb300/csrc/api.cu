@@ -258,7 +258,7 @@ lbm_status sweep_step(const lbm_plan* p, const void* src, void* dst, const Bc& b
                       cudaStream_t s, const PlanInfo* info = nullptr)
 {
     if (!in_place(p)) return step_launch(info ? *info : p->info, kStreamCollide, src, dst, at_time(bc, t), tau, s);
-    return step_launch_cmp(p->info, kStreamCollide, src, dst, false, false, at_time(bc, t), tau, s,
+    return step_launch_cmp(p->info, kStreamCollide, src, dst, at_time(bc, t), tau, s,
                            layout_at(true, t - 1), layout_at(true, t));
 }
 
@@ -704,7 +704,7 @@ lbm_status lbm_step(lbm_plan* p, const double* d_rho_in, const double* d_tau, do
     Bc bcs = bc;
     if (one) bcs.side_u = ws + p->ws.side;  // the collide-only launch writes the Eq. 6 nodes' velocities
     if (p->info.cmp.nf)
-        LBM_TRY(step_launch_cmp(p->info, kCollideOnly, d_f_in, ping0, true, false, bcs, tau, s));
+        LBM_TRY(step_launch_cmp(p->info, kCollideOnly, d_f_in, ping0, bcs, tau, s));
     else
         LBM_TRY(step_launch(p->info, kCollideOnly, d_f_in, ping0, bc, tau, s));
     // n - 1 stream-collide steps, two per launch where the two-step kernel applies

@@ -693,7 +693,7 @@ lbm_status lbm_batch_forward(lbm_batch* b, const double* d_rho_in, const double*
         for (int t = 1; t <= T - 1; ++t) {
             unsigned char* dst = slot(t);
             if (!dst) dst = ws + b->o_ping[t & 1];
-            lbm_status st = b->cmp ? bstep_launch_cmp(ca, kStreamCollide, cur, dst, false, d_rho_in, d_tau, rho_out, st_)
+            lbm_status st = b->cmp ? bstep_launch_cmp(ca, kStreamCollide, cur, dst, d_rho_in, d_tau, rho_out, st_)
                                    : step(b, kStreamCollide, cur, dst, d_rho_in, d_tau, rho_out, ws, st_);
             if (st != LBM_OK) return st;
             cur = dst;
@@ -701,7 +701,7 @@ lbm_status lbm_batch_forward(lbm_batch* b, const double* d_rho_in, const double*
         if (!b->cmp) return step(b, kStreamOnly, cur, d_f, d_rho_in, d_tau, rho_out, ws, st_);
         // fluid nodes only: the solid entries of the caller's packed array are zeroed first
         if (cudaMemsetAsync(d_f, 0, (size_t)b->state_elems * (size_t)b->prec, st_) != cudaSuccess) return LBM_ERR_CUDA;
-        return bstep_launch_cmp(ca, kStreamOnly, cur, d_f, true, d_rho_in, d_tau, rho_out, st_);
+        return bstep_launch_cmp(ca, kStreamOnly, cur, d_f, d_rho_in, d_tau, rho_out, st_);
     };
     return run_graph(b, b->cmp ? 11 : 1, {d_rho_in, d_tau, d_f, d_ws}, rho_out, s, issue);
 }
@@ -781,7 +781,7 @@ lbm_status lbm_batch_adjoint(lbm_batch* b, const double* d_rho_in, const double*
                     if (cudaMemsetAsync(seg(1), 0, sb, st_) != cudaSuccess) return LBM_ERR_CUDA;
                 } else {
                     lbm_status st =
-                        b->cmp ? bstep_launch_cmp(ca, kStreamCollide, prev, seg(j), false, d_rho_in, d_tau, rho_out, st_)
+                        b->cmp ? bstep_launch_cmp(ca, kStreamCollide, prev, seg(j), d_rho_in, d_tau, rho_out, st_)
                                : step(b, kStreamCollide, prev, seg(j), d_rho_in, d_tau, rho_out, ws, st_);
                     if (st != LBM_OK) return st;
                 }

@@ -344,8 +344,8 @@ struct BCmpArgs {
     int q, prec, pdl;
     uint32_t* status;
 };
-lbm_status bstep_launch_cmp(const BCmpArgs& a, int mode, const void* src, void* dst, bool dense_out,
-                            const double* rho_in, const double* tau, double rho_out, cudaStream_t s);
+lbm_status bstep_launch_cmp(const BCmpArgs& a, int mode, const void* src, void* dst, const double* rho_in,
+                            const double* tau, double rho_out, cudaStream_t s);
 lbm_status badjoint_launch_cmp(const BCmpArgs& a, int t0, const void* gprev, const void* lam_in, void* lam_out,
                                const double* rho_in, const double* tau, double rho_out, double* grad_acc,
                                double* partial, cudaStream_t s);
@@ -368,10 +368,9 @@ constexpr int kLayoutSwapped = 1;
 // The layout of g^t (and lambda^t) in a sweep of the in-place schedule.
 inline int layout_at(bool aa, long long t) { return aa && (t & 1) ? kLayoutSwapped : kLayoutNatural; }
 // lin / lout: layouts of the input and output states (stream-collide: natural -> natural is the two-buffer pull,
-// natural -> swapped and swapped -> natural the in-place pair; stream-only into the caller's array: any lin)
-lbm_status step_launch_cmp(const PlanInfo& p, int mode, const void* src, void* dst, bool dense_in, bool dense_out,
-                           const Bc& bc, const double* tau, cudaStream_t s, int lin = kLayoutNatural,
-                           int lout = kLayoutNatural);
+// natural -> swapped and swapped -> natural the in-place pair); collide-only reads the caller's dense array
+lbm_status step_launch_cmp(const PlanInfo& p, int mode, const void* src, void* dst, const Bc& bc, const double* tau,
+                           cudaStream_t s, int lin = kLayoutNatural, int lout = kLayoutNatural);
 // stream-only from a compact state into the caller's dense array, every entry written (solid nodes zero)
 lbm_status stream_dense_launch(const PlanInfo& p, const void* src, void* dst, const Bc& bc, cudaStream_t s,
                                int lin = kLayoutNatural);

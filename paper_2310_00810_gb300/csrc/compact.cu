@@ -758,7 +758,7 @@ __device__ __forceinline__ void keep_velocity(const T (&v)[Q], const Side& sd, c
 // columns (the last ones of a lattice), whose update is the longest, first;
 // then the interior, upwards or (rev) downwards.  Alternating the direction
 // from launch to launch starts each launch on what the one before left in
-// the L2 cache.
+// the L2 cache (a batch's launches carry no time level and all go upwards).
 struct CmpOrder {
     unsigned n, first;  // node blocks; how many of the last come first
     int rev;
@@ -966,9 +966,9 @@ constexpr int kMinBlocks = sizeof(T) == 8 ? 2 : 4;
 // beside it (D3Q19 512x256x256: step 549 -> 469 us, adjoint 874 -> 833 us of
 // kernel time; D2Q9: see the pipelined forms).
 
-// One step.  MODE: stream-collide, collide-only or stream-only (step.cu);
-// DIN: the collide-only input is the instance's dense [Q][N] array; IN / OUT:
-// the addressing of the input and output states (two-buffer pull: gather /
+// One step.  MODE: stream-collide, collide-only (from the instance's dense
+// [Q][N] array) or stream-only (step.cu); IN / OUT: the addressing of the
+// input and output states (two-buffer pull: gather /
 // own; in place: gather / scatter, then local / own; OUT dense: the caller's
 // array, solid entries left to the caller).  src == dst is allowed for the
 // in-place pairs: the slot sets of different nodes are disjoint, and a node
@@ -979,7 +979,7 @@ constexpr int kMinBlocks = sizeof(T) == 8 ? 2 : 4;
 // for the preceding launch, or (in place) hit a line that another block has
 // rewritten since.  Padding nodes of a batch are skipped: nothing ever reads
 // them.
-template <int Q, typename T, int MODE, bool DIN, int IN, int OUT, bool DENSE_ROUND>
+template <int Q, typename T, int MODE, int IN, int OUT, bool DENSE_ROUND>
 __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
     k_step_cmp(const T* src, T* dst, Cmp c, CmpBlk lat, const BCmpInst* __restrict__ insts,
                const CmpBlk* __restrict__ blks, Bc tmpl, const double* __restrict__ tau, CmpOrder ord)
@@ -998,8 +998,8 @@ __global__ void __launch_bounds__(kCmpThreads, kMinBlocks<T>)
     if (MODE == kCollideOnly) {
         if (side && eq6_bit(c, k)) wall.sd = side_of(c.idx, k, I->g);
         pdl_enter();
-        const T* s = DIN ? src + I->f_off + c.idx[k] : src + k;
-        const size_t S = DIN ? (size_t)I->g.N : (size_t)c.nf;
+        const T* s = src + I->f_off + c.idx[k];
+        const size_t S = (size_t)I->g.N;
 #pragma unroll
         for (int i = 0; i < Q; ++i) v[i] = s[(size_t)i * S];
     } else if (!nd.bnd()) {
@@ -1396,9 +1396,9 @@ BCmpArgs single_args(const PlanInfo& p, uint32_t* status)
 
 // The sweeps use: stream-collide compact -> compact (two-buffer pull
 // natural -> natural, or the in-place pair natural -> swapped, swapped ->
-// natural); collide-only from a dense or compact state into compact;
-// stream-only into compact or into the caller's dense array, from either
-// layout.
+// natural); collide-only from the caller's dense array into compact;
+// stream-only into the caller's dense array (batches from here, by compact
+// node; single lattices through k_stream_dense).
 // Threads per block of the one-node-per-thread kernels.  Below one wave small
 // blocks spread the few warps evenly over the SMs (128x64 to 512x256 D2Q9:
 // 64 threads 6.3 to 7.7 us per time step of a gradient evaluation, 256
@@ -1411,9 +1411,11 @@ unsigned cmp_threads(int q, int prec, long long nf)
     return q == 9 ? 128 : 256;
 }
 
-// The pipelined kernels, from four nodes per resident thread: D2Q9 FP32
-// 2048x1024 takes 58.9 us per time step of a gradient evaluation with them
-// and 71.5 with one node per thread, 1024x512 17.6 and 16.6.  D3Q19 stays
+// The pipelined kernels, from 600000 nodes (6 to 8 per resident thread at 4
+// and 5 CTAs on each of 152 SMs; the line lies between two measured sizes):
+// D2Q9 FP32 2048x1024, 1.3 M fluid nodes, takes 58.9 us per time step of a
+// gradient evaluation with them and 71.5 with one node per thread, 1024x512,
+// 0.3 M, 17.6 and 16.6.  D3Q19 stays
 // with one node per thread: two nodes' populations in registers leave 16
 // warps per SM (512x256x256: 1829 us per step, pipelined 2085).
 template <int Q, typename T>
@@ -1450,8 +1452,8 @@ CmpOrder pipe_order(const BCmpArgs& a, int t)
 }
 
 template <int Q, typename T, bool DENSE_ROUND>
-void launch_step_as(const BCmpArgs& a, int mode, const void* src, void* dst, bool din, bool dout, int lin, int lout,
-                 const Bc& tmpl, const double* tau, cudaStream_t s)
+void launch_step_as(const BCmpArgs& a, int mode, const void* src, void* dst, int lin, int lout, const Bc& tmpl,
+                    const double* tau, cudaStream_t s)
 {
     const T* x = static_cast<const T*>(src);
     T* y = static_cast<T*>(dst);
@@ -1459,12 +1461,12 @@ void launch_step_as(const BCmpArgs& a, int mode, const void* src, void* dst, boo
     const CmpOrder ord = cmp_order(a, threads, tmpl.t_level);
     const dim3 grid(ord.n), block(threads);
     const bool swap_in = lin == kLayoutSwapped, swap_out = lout == kLayoutSwapped;
-    auto go = [&](auto kernel, dim3 gr) {
-        launch_k(a.pdl, kernel, gr, block, 0, s, x, y, a.c, a.lat, a.insts, a.blks, tmpl, tau, ord);
+    auto go = [&](auto kernel) {
+        launch_k(a.pdl, kernel, grid, block, 0, s, x, y, a.c, a.lat, a.insts, a.blks, tmpl, tau, ord);
     };
     if (mode == kStreamCollide) {
         if (swap_in) {  // the local step: its interior nodes read their own slots
-            go(k_step_cmp<Q, T, kStreamCollide, false, kInLocal, kOutOwn, DENSE_ROUND>, grid);
+            go(k_step_cmp<Q, T, kStreamCollide, kInLocal, kOutOwn, DENSE_ROUND>);
             return;
         }
         if constexpr (kPipe<Q, T>) {
@@ -1477,32 +1479,26 @@ void launch_step_as(const BCmpArgs& a, int mode, const void* src, void* dst, boo
                 return;
             }
         }
-        if (swap_out) go(k_step_cmp<Q, T, kStreamCollide, false, kInGather, kOutScatter, DENSE_ROUND>, grid);
-        else go(k_step_cmp<Q, T, kStreamCollide, false, kInGather, kOutOwn, DENSE_ROUND>, grid);
-    } else if (mode == kCollideOnly && din) {
-        go(k_step_cmp<Q, T, kCollideOnly, true, kInGather, kOutOwn, DENSE_ROUND>, grid);
+        if (swap_out) go(k_step_cmp<Q, T, kStreamCollide, kInGather, kOutScatter, DENSE_ROUND>);
+        else go(k_step_cmp<Q, T, kStreamCollide, kInGather, kOutOwn, DENSE_ROUND>);
     } else if (mode == kCollideOnly) {
-        go(k_step_cmp<Q, T, kCollideOnly, false, kInGather, kOutOwn, DENSE_ROUND>, grid);
-    } else if (dout && swap_in) {
-        go(k_step_cmp<Q, T, kStreamOnly, false, kInLocal, kOutDense, DENSE_ROUND>, grid);
-    } else if (dout) {
-        go(k_step_cmp<Q, T, kStreamOnly, false, kInGather, kOutDense, DENSE_ROUND>, grid);
+        go(k_step_cmp<Q, T, kCollideOnly, kInGather, kOutOwn, DENSE_ROUND>);
     } else {
-        go(k_step_cmp<Q, T, kStreamOnly, false, kInGather, kOutOwn, DENSE_ROUND>, grid);
+        go(k_step_cmp<Q, T, kStreamOnly, kInGather, kOutDense, DENSE_ROUND>);
     }
 }
 
 template <int Q, typename T>
-void launch_step(const BCmpArgs& a, int mode, const void* src, void* dst, bool din, bool dout, int lin, int lout,
-                 const Bc& tmpl, const double* tau, cudaStream_t s)
+void launch_step(const BCmpArgs& a, int mode, const void* src, void* dst, int lin, int lout, const Bc& tmpl,
+                 const double* tau, cudaStream_t s)
 {
     if constexpr (Q == 9 && std::is_same<T, float>::value) {
         if (a.dense_round && mode != kStreamOnly) {
-            launch_step_as<Q, T, true>(a, mode, src, dst, din, dout, lin, lout, tmpl, tau, s);
+            launch_step_as<Q, T, true>(a, mode, src, dst, lin, lout, tmpl, tau, s);
             return;
         }
     }
-    launch_step_as<Q, T, false>(a, mode, src, dst, din, dout, lin, lout, tmpl, tau, s);
+    launch_step_as<Q, T, false>(a, mode, src, dst, lin, lout, tmpl, tau, s);
 }
 
 template <int Q, typename T, int IN, int OUT, bool DENSE_ROUND>
@@ -1556,14 +1552,14 @@ void launch_adjoint(const BCmpArgs& a, int t0, const void* gprev, const void* la
     as(std::false_type{});
 }
 
-lbm_status step_any(const BCmpArgs& a, int mode, const void* src, void* dst, bool din, bool dout, const Bc& tmpl,
-                    const double* tau, cudaStream_t s, int lin = kLayoutNatural, int lout = kLayoutNatural)
+lbm_status step_any(const BCmpArgs& a, int mode, const void* src, void* dst, const Bc& tmpl, const double* tau,
+                    cudaStream_t s, int lin = kLayoutNatural, int lout = kLayoutNatural)
 {
     if (a.n_blocks == 0) return LBM_OK;
-    if (a.q == 9 && a.prec == 4) launch_step<9, float>(a, mode, src, dst, din, dout, lin, lout, tmpl, tau, s);
-    else if (a.q == 9 && a.prec == 8) launch_step<9, double>(a, mode, src, dst, din, dout, lin, lout, tmpl, tau, s);
-    else if (a.q == 19 && a.prec == 4) launch_step<19, float>(a, mode, src, dst, din, dout, lin, lout, tmpl, tau, s);
-    else if (a.q == 19 && a.prec == 8) launch_step<19, double>(a, mode, src, dst, din, dout, lin, lout, tmpl, tau, s);
+    if (a.q == 9 && a.prec == 4) launch_step<9, float>(a, mode, src, dst, lin, lout, tmpl, tau, s);
+    else if (a.q == 9 && a.prec == 8) launch_step<9, double>(a, mode, src, dst, lin, lout, tmpl, tau, s);
+    else if (a.q == 19 && a.prec == 4) launch_step<19, float>(a, mode, src, dst, lin, lout, tmpl, tau, s);
+    else if (a.q == 19 && a.prec == 8) launch_step<19, double>(a, mode, src, dst, lin, lout, tmpl, tau, s);
     else return LBM_ERR_UNSUPPORTED;
     return cuda_status(cudaGetLastError());
 }
@@ -1712,11 +1708,11 @@ lbm_status compact_build(const PlanInfo& p, long long nf, void* tables, Cmp* out
     return LBM_OK;
 }
 
-lbm_status step_launch_cmp(const PlanInfo& p, int mode, const void* src, void* dst, bool dense_in, bool dense_out,
-                           const Bc& bc, const double* tau, cudaStream_t s, int lin, int lout)
+lbm_status step_launch_cmp(const PlanInfo& p, int mode, const void* src, void* dst, const Bc& bc,
+                           const double* tau, cudaStream_t s, int lin, int lout)
 {
     if (p.cmp.nf == 0) return LBM_OK;
-    return step_any(single_args(p, bc.status), mode, src, dst, dense_in, dense_out, bc, tau, s, lin, lout);
+    return step_any(single_args(p, bc.status), mode, src, dst, bc, tau, s, lin, lout);
 }
 
 template <int Q, typename T>
@@ -1783,10 +1779,10 @@ lbm_status compact_gather_add_launch(const PlanInfo& p, const void* dense, void*
     return gather_any(single_args(p, nullptr), dense, compact, s, true, layout);
 }
 
-lbm_status bstep_launch_cmp(const BCmpArgs& a, int mode, const void* src, void* dst, bool dense_out,
-                            const double* rho_in, const double* tau, double rho_out, cudaStream_t s)
+lbm_status bstep_launch_cmp(const BCmpArgs& a, int mode, const void* src, void* dst, const double* rho_in,
+                            const double* tau, double rho_out, cudaStream_t s)
 {
-    return step_any(a, mode, src, dst, false, dense_out, batch_tmpl(rho_in, rho_out, a.status), tau, s);
+    return step_any(a, mode, src, dst, batch_tmpl(rho_in, rho_out, a.status), tau, s);
 }
 
 lbm_status badjoint_launch_cmp(const BCmpArgs& a, int t0, const void* gprev, const void* lam_in, void* lam_out,

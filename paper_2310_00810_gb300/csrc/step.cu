@@ -78,7 +78,7 @@ static void launch(const PlanInfo& p, int mode, const void* src, void* dst, cons
 lbm_status step_launch(const PlanInfo& plan, int mode, const void* src, void* dst, const Bc& bc, const double* tau,
                        cudaStream_t s)
 {
-    if (plan.cmp.nf) return step_launch_cmp(plan, mode, src, dst, false, false, bc, tau, s);
+    if (plan.cmp.nf) return step_launch_cmp(plan, mode, src, dst, bc, tau, s);
     // the extrapolated Eq. 6 velocity and the MRT collision are implemented by the one-node-per-thread kernels
     const int family = bc.uw_extrap || bc.mrt || auto_scalar(plan, plan.step_family) ? LBM_FAMILY_SCALAR
                                                                                      : plan.step_family;

@@ -1041,8 +1041,8 @@ __global__ void __launch_bounds__(128, 1) k_umma_wgrad(const __grid_constant__ C
 // 50 us: every kernel is launched with programmatic stream serialization and
 // waits for its predecessor itself, so a launch's setup overlaps the one
 // before, and what a pass would only mask, copy or convert is done where the
-// values are written (2463 -> 1930 us per step, prediction of one field 337
-// -> 210 us).
+// values are written (2463 -> 1930 us per step, prediction of one field 337 ->
+// 210 us; with the input layer's kernels and the rings by grid 1768 and 177).
 
 // out[i] = sum over splits of part[split * stride + i], in order.  Few outputs
 // of many splits take one warp each, lane l adding splits l, l + 32, ... in
@@ -1461,6 +1461,7 @@ std::vector<Tensor> param_tensors(int base, std::vector<int>* taps_out = nullptr
 }
 
 constexpr int kMaxSplits = 256;
+constexpr int kColsumBlocks = 608;  // blocks of a column sum, at most: four on each of 152 SMs
 constexpr long long kTargetCtas = 608;  // weight-gradient CTAs aimed for (4 per SM)
 
 struct Layout {
@@ -1553,7 +1554,7 @@ bool make_layout(const unet_desc* d, Layout* L)
     l.part_floats = max_part;
     o += al256(sizeof(float) * (size_t)max_part);
     l.part_b = o;
-    o += al256(sizeof(float) * 608 * (size_t)(2 * l.c[3]));
+    o += al256(sizeof(float) * kColsumBlocks * (size_t)(2 * l.c[3]));
     l.total = o;
     return true;
 }
@@ -1757,8 +1758,7 @@ int umma_wgrad(cudaStream_t s, const bf16* x, int Bimg, int H, int W, int Cin, i
     return ok ? (int)sp : 0;
 }
 
-// Rows per block of a column sum: four blocks per SM, at least 64 rows each.
-constexpr int kColsumBlocks = 608;
+// Rows per block of a column sum, at least 64.
 long long colsum_rows(long long P) { return std::max(64LL, (P + kColsumBlocks - 1) / kColsumBlocks); }
 
 // Whether the input layer's own kernels take a convolution.
