@@ -58,7 +58,7 @@ def parse():
                     help="--mode unet: the convolutions' GEMM engine")
     ap.add_argument("--lattice", default="disks8192x4096", help="workload name for --mode kernels")
     ap.add_argument("--layout", default=None, choices=[None, "dense", "compact"],
-                    help="state layout for --mode kernels (default: compact for D3Q19, dense for D2Q9)")
+                    help="state layout for --mode kernels (default: compact)")
     ap.add_argument("--launches", type=int, default=20)
     ap.add_argument("--aa", type=int, default=0, choices=[0, 1],
                     help="--mode kernels: the in-place (AA-pattern) schedule of the fluid-only layout")
@@ -575,7 +575,7 @@ def learned_init_leg(device, n_train, epochs, n_eval, time_limit):
     zero_single = float(np.mean([r["zero"]["seconds"] for r in rows]))
     mean = lambda key, f: float(np.mean([f(r[key]) for r in rows]))
     return {"workload": f"U-Net base {base}, input 2 velocity channels + mask at {nx}x{ny}, BF16 weights/activations, "
-                        f"FP32 accumulation (mma.sync tensor cores); {n_train} training solves (D2Q9 FP32, T={T}, "
+                        f"FP32 accumulation (tcgen05 tensor cores); {n_train} training solves (D2Q9 FP32, T={T}, "
                         f"disks r 6-12, porosity U[0.5, 0.7], seeds 5000+j), {epochs} epochs, held-out seeds 25000+i",
             "generation_s": round(t_gen, 2), "solves_per_s": round(n_train / t_gen, 2),
             "train_s": round(t_train, 2), "train_samples_per_s": round(samples / t_train, 1),
@@ -776,10 +776,10 @@ def run_e2e(P, args, device, barrier, world):
 HBM_TRAFFIC = {
     ("disks8192x4096", "dense"): {"stream-collide": 4 * (343.118080e6 + 201.248512e6),
                                   "adjoint": 4 * (642.651648e6 + 217.033472e6)},
-    ("disks8192x4096", "compact"): {"stream-collide": 20132542 / 5032998 * (343.8e6 + 144.4e6),
-                                    "adjoint": 20132542 / 5032998 * (527.8e6 + 158.9e6)},
-    ("spheres512x256x256", "compact"): {"stream-collide": 15090843 / 1886221 * (297.2e6 + 112.1e6),
-                                        "adjoint": 15090843 / 1886221 * (463.7e6 + 130.9e6)},
+    ("disks8192x4096", "compact"): {"stream-collide": 20132542 / 5032998 * (205.4e6 + 133.6e6),
+                                    "adjoint": 20132542 / 5032998 * (389.4e6 + 151.0e6)},
+    ("spheres512x256x256", "compact"): {"stream-collide": 15090843 / 1886221 * (170.5e6 + 94.4e6),
+                                        "adjoint": 15090843 / 1886221 * (335.5e6 + 116.6e6)},
 }
 
 

@@ -512,8 +512,9 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm(LA la, LB lb, EP ep, long
 // short a row for the tensor-memory kernels' boxes, and K = 72.  Both of its
 // products move little more than its output (33 MB at 256 x 128, batch 16,
 // base 32), so these kernels feed mma.sync straight from memory, without the
-// general gather's index arithmetic: forward 72 -> 12 us, weight gradient
-// 93 -> 17 us.
+// general gather's index arithmetic: forward 72 -> 34 us, weight gradient
+// 93 -> 35 us (a launch alone, warm; bound by issue and by latency: the tensor
+// pipe is 13 % active, DRAM 3 and 14 % of its rate).
 
 // y = relu(conv3x3(x) + bias): a warp takes 16 pixels of a row x 32 output
 // channels; an A fragment's registers are 4-byte loads (two channels of a
