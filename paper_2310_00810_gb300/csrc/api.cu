@@ -481,8 +481,10 @@ lbm_status lbm_set_collision(lbm_plan* p, int32_t mode, double s_e, double s_eps
 lbm_status lbm_set_rounding(lbm_plan* p, int32_t mode)
 {
     if (!p || mode < LBM_ROUND_NATIVE || mode > LBM_ROUND_DENSE_NODE) return LBM_ERR_INVALID_ARG;
-    p->info.dense_round = mode == LBM_ROUND_DENSE ? 1 : 0;
-    p->info.node_round = mode == LBM_ROUND_DENSE_NODE ? 1 : 0;
+    const int dense = mode == LBM_ROUND_DENSE ? 1 : 0, node = mode == LBM_ROUND_DENSE_NODE ? 1 : 0;
+    if (p->info.dense_round == dense && p->info.node_round == node) return LBM_OK;  // the captured sweeps stay
+    p->info.dense_round = dense;
+    p->info.node_round = node;
     drop_graphs(p);
     return LBM_OK;
 }

@@ -1,4 +1,6 @@
 """The automatic layout of D2Q9 solvers against calls that change it or its kernels."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -173,3 +175,28 @@ def test_tuning_results_are_kept_apart_by_what_decides_them(tmp_path):
     assert not autotune.tune(mrt, t_tune=8, repeats=1, cache=cache)["cached"]
     opened = lbm.Solver(9, 65, 41, n_steps=30, inlet_kind=lbm.LBM_INLET_PROFILE, geometry=_mask(65, 41, solid=0.0))
     assert not autotune.tune(opened, t_tune=8, repeats=1, cache=cache)["cached"]
+
+
+@pytest.mark.parametrize("layout", ["dense", "compact"])
+def test_naming_the_layout_it_has_keeps_the_captured_sweeps(layout):
+    """A sweep after it costs the host a replay, not a capture of thousands of launches (milliseconds)."""
+    s = _solver(T=6000, layout=layout)
+    p, _ = _inputs(s)
+    f = s.new_state()
+
+    def host_ms():
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        s.forward(*p, f)
+        dt = (time.perf_counter() - t0) * 1e3
+        torch.cuda.synchronize()
+        return dt
+
+    def again():
+        s.set_layout(layout)
+        return host_ms()
+
+    first = host_ms()
+    same = min(host_ms() for _ in range(3))
+    assert first > 2.0
+    assert min(again() for _ in range(3)) < max(5 * same, 1.5)
