@@ -564,6 +564,8 @@ class Solver:
         needs another forward sweep first).  On a D2Q9 lattice in the automatic
         layout that holds the checkpoints of a forward sweep, "dense" takes
         effect at the next forward(): the reverse sweep may still follow."""
+        if layout not in ("dense", "compact"):
+            raise ValueError(f"layout must be dense or compact, not {layout!r}")
         p = self.plan
         auto, self._auto_2d = self._auto_2d, False
         self._next_dense = (auto or self._next_dense) and layout == "dense" and p._swept and self._bound == "compact"
@@ -585,10 +587,8 @@ class Solver:
             tables = torch.empty(max(lbm_compact_size(p, nf), 256), dtype=torch.uint8, device=self.device)
             self.run(lambda: lbm_compact_bind(p, nf, tables, self.stream))
             self.n_fluid = nf
-        elif layout == "dense":
-            self.run(lambda: lbm_compact_bind(p, 0, None, self.stream))
         else:
-            raise ValueError(f"layout must be dense or compact, not {layout!r}")
+            self.run(lambda: lbm_compact_bind(p, 0, None, self.stream))
         p._swept = False
         self.ws = torch.zeros(lbm_workspace_size(p), dtype=torch.uint8, device=self.device)
 

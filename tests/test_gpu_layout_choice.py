@@ -200,3 +200,16 @@ def test_naming_the_layout_it_has_keeps_the_captured_sweeps(layout):
     same = min(host_ms() for _ in range(3))
     assert first > 2.0
     assert min(again() for _ in range(3)) < max(5 * same, 1.5)
+
+
+def test_a_refused_choice_changes_nothing():
+    s = _solver()
+    want = _gradient(s)
+    with pytest.raises(ValueError):
+        s.set_layout("sparse")
+    with pytest.raises(lbm.LBMError):
+        s.set_kernels(step_family=9)
+    assert s.layout == "compact" and _same(_gradient(s), want)
+    s.set_kernels(step_family=lbm.LBM_FAMILY_VEC)  # the layout is still automatic
+    s.forward(*_inputs(s)[0])
+    assert s.layout == "dense"
